@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "capi_internal.h"
+#include "mixed_plans.h"
 #include "roots.cuh"
 
 namespace fft3 {
@@ -27,6 +28,17 @@ extern const FixedKernels g_fixed_kernels_a[];
 extern const int g_fixed_kernels_a_count;
 extern const FixedKernels g_fixed_kernels_b[];
 extern const int g_fixed_kernels_b_count;
+
+extern const MixedKernels g_mixed_kernels_a[], g_mixed_kernels_b[], g_mixed_kernels_c[], g_mixed_kernels_d[];
+
+const MixedKernels *mixed_kernels(int n)
+{
+    for (const MixedKernels *t : {g_mixed_kernels_a, g_mixed_kernels_b, g_mixed_kernels_c, g_mixed_kernels_d})
+        for (; t->n; ++t)
+            if (t->n == n)
+                return t;
+    return nullptr;
+}
 
 const FixedKernels *fixed_kernels(int id)
 {
@@ -262,7 +274,11 @@ static int build_launches(fft3_plan_s *P)
             L.func = fk ? fk->ctma : nullptr;
             L.tma = true;
             break;
-        case PK_G: L.func = (const void *)&k_pass_g; break;
+        case PK_G: {
+            const MixedKernels *mk = p.mixed ? mixed_kernels(p.line.n) : nullptr;
+            L.func = !p.mixed ? (const void *)&k_pass_g : mk ? (p.mixed == 1 ? mk->j : mk->c) : nullptr;
+            break;
+        }
         case PK_G64: L.func = (const void *)&k_pass_g64; break;
         case PK_J64:
         case PK_C64: {

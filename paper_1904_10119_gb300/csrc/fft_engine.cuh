@@ -348,25 +348,50 @@ __host__ __device__ constexpr double sin10(int m)
                                                                                         : -kS72;
 }
 
-// a * w_N^M for N in {6, 10, 12} (and the powers of two of mul_w), M known at
-// compile time.
+// cos and sin of 2 pi m / 9 and 2 pi m / 15 for m <= N/2.
+constexpr double kCos9[5] = {
+    1.000000000000000000000000000000000000, 0.766044443118978035202392650555416674,
+    0.173648177666930348851716626769314796, -0.500000000000000000000000000000000000,
+    -0.939692620785908384054109277324731470};
+constexpr double kSin9[5] = {
+    0E-36, 0.642787609686539326322643409907263433,
+    0.984807753012208059366743024589523014, 0.866025403784438646763723170752936183,
+    0.342020143325668733044099614682259581};
+constexpr double kCos15[8] = {
+    1.000000000000000000000000000000000000, 0.913545457642600895502127571985317178,
+    0.669130606358858213826273330686780474, 0.309016994374947424102293417182819059,
+    -0.104528463267653471399834154802498119, -0.500000000000000000000000000000000000,
+    -0.809016994374947424102293417182819059, -0.978147600733805637928566747869599532};
+constexpr double kSin15[8] = {
+    0E-36, 0.406736643075800207753985990341497613,
+    0.743144825477394235014697048974256977, 0.951056516295153572116439333379382143,
+    0.994521895368273336922691944980570382, 0.866025403784438646763723170752936183,
+    0.587785252292473129168705954639072769, 0.207911690817759337101742284405125166};
+__host__ __device__ constexpr double cos9(int m) { return m <= 4 ? kCos9[m] : kCos9[9 - m]; }
+__host__ __device__ constexpr double sin9(int m) { return m <= 4 ? kSin9[m] : -kSin9[9 - m]; }
+__host__ __device__ constexpr double cos15(int m) { return m <= 7 ? kCos15[m] : kCos15[15 - m]; }
+__host__ __device__ constexpr double sin15(int m) { return m <= 7 ? kSin15[m] : -kSin15[15 - m]; }
+
+// a * w_N^M for N in {6, 9, 10, 12, 15} (and the powers of two of mul_w), M
+// known at compile time.
 template <int N, int M, class C>
 __device__ __forceinline__ C mul_wn(C a)
 {
     if constexpr (16 % N == 0) {
         return mul_w<N, M>(a);
     } else {
-        static_assert(N == 6 || N == 10 || N == 12, "composite twiddles exist for 6, 10 and 12 points");
+        static_assert(N == 6 || N == 9 || N == 10 || N == 12 || N == 15,
+                      "composite twiddles exist for 6, 9, 10, 12 and 15 points");
         using X = Cx<C>;
         using S = typename X::S;
         constexpr int m = ((M % N) + N) % N;
         if constexpr (m == 0) {
             return a;
-        } else if constexpr (N != 10 && (m * (12 / N)) % 3 == 0) {
+        } else if constexpr (12 % N == 0 && (m * (12 / N)) % 3 == 0) {
             return mul_w<4, (m * (12 / N)) / 3>(a); // multiples of 90 degrees
         } else {
-            constexpr S c = (S)(N == 10 ? cos10(m) : cos12(m * (12 / N)));
-            constexpr S s = (S)(N == 10 ? sin10(m) : sin12(m * (12 / N)));
+            constexpr S c = (S)(N == 9 ? cos9(m) : N == 15 ? cos15(m) : N == 10 ? cos10(m) : cos12(m * (12 / N)));
+            constexpr S s = (S)(N == 9 ? sin9(m) : N == 15 ? sin15(m) : N == 10 ? sin10(m) : sin12(m * (12 / N)));
             return X::make(X::fma_(a.x, c, a.y * s), X::fma_(a.y, c, -a.x * s));
         }
     }
@@ -422,6 +447,10 @@ template <>
 struct Bfly<10> : BflyCt<2, 5> {};
 template <>
 struct Bfly<12> : BflyCt<4, 3> {};
+template <>
+struct Bfly<9> : BflyCt<3, 3> {};
+template <>
+struct Bfly<15> : BflyCt<3, 5> {};
 
 // ------------------------------------------------------ stage indexing -- //
 // Shared-memory position of intra-line index `pos` for the line-major layout:

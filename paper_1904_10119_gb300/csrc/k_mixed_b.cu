@@ -1,0 +1,6 @@
+// Mixed-radix line passes, part B of the plan list.
+#include "k_mixed.cuh"
+
+namespace fft3 {
+extern const MixedKernels g_mixed_kernels_b[] = {FFT3_MIXED_PLANS_B(FFT3_MIXED_ROW){0, nullptr, nullptr}};
+} // namespace fft3

@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <sstream>
 
+#include "mixed_plans.h"
 #include "plans.h"
 #include "roots.cuh"
 
@@ -72,6 +73,18 @@ const CStreamKernel *cstream_meta(int *count)
 {
     *count = (int)(sizeof(g_cstream_meta) / sizeof(g_cstream_meta[0]));
     return g_cstream_meta;
+}
+
+#define FFT3_MIXED_META(N, T, ...) {N, T, {__VA_ARGS__}},
+static const MixedPlanMeta g_mixed_meta[] = {FFT3_MIXED_PLANS(FFT3_MIXED_META)};
+#undef FFT3_MIXED_META
+
+static const MixedPlanMeta *mixed_plan(int n)
+{
+    for (const MixedPlanMeta &m : g_mixed_meta)
+        if (m.n == n)
+            return &m;
+    return nullptr;
 }
 
 int fixed_plan_count() { return g_nmeta; }
@@ -523,9 +536,23 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
         }
         p.kind = PK_G;
     }
+    // lines of a mixed plan's length, contiguous on both sides or strided columns:
+    // the compile-time passes (k_mixed.cuh) under the default radix order; the
+    // rotated store and radix orders 1..3 keep the runtime lists
+    const MixedPlanMeta *mp = p.kind == PK_G && order == 0 && !rotate && g.oblk == 0 ? mixed_plan(n) : nullptr;
+    if (mp && ((contig_in && g.ok == 1) || strided_in)) {
+        p.mixed = contig_in && g.ok == 1 ? 1 : 2;
+        p.line.T = mp->T;
+        for (p.line.nst = 0; p.line.nst < 8 && mp->rad[p.line.nst] > 0; ++p.line.nst)
+            p.line.rad[p.line.nst] = mp->rad[p.line.nst];
+    }
     p.tw_seg[0] = line_seg(s, p.line);
     int tw_len = (int)s->tw[p.tw_seg[0]].m.size();
-    if (p.kind == PK_G) {
+    if (p.mixed) {
+        p.lpt = p.mixed == 1 ? lpt_j(p.line.T) : mixed_lpt_c(n, p.line.T);
+        p.threads = p.line.T * p.lpt;
+        p.smem_bytes = (tw_slots_h(tw_len) + p.lpt * (p.mixed == 1 ? pitch_h(n) : n)) * 8;
+    } else if (p.kind == PK_G) {
         generic_launch_shape(n, p.line.T, !contig_in, tw_len, &p.lpt, &p.threads, &p.smem_bytes);
     } else if (p.kind == PK_J) {
         p.threads = p.line.T * p.lpt;
@@ -1470,6 +1497,8 @@ std::string Schedule::json() const
             o << ",\"q\":" << m.q << ",\"m\":" << m.n / m.q << ",\"groups\":" << m.groups
               << ",\"staging\":" << m.groups * m.stages << ",\"cluster\":" << m.pair;
         }
+        if (p.mixed)
+            o << ",\"compiled\":true";
         if (p.chunk > 0)
             o << ",\"chunk\":" << p.chunk << ",\"pipelined_with\":\"" << (p.pair_next ? "next" : "previous")
               << "\"";
