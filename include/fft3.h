@@ -48,9 +48,11 @@ enum fft3_dtype {
     FFT3_C64_SPLITBF16_TC = 1, /* radix-32 / radix-16 sub-DFTs as split-BF16 tensor-core GEMMs (hi + lo
                                   BF16 parts, three products), FP32 accumulation (options.tc_stages) */
     FFT3_C128_FP64 = 2         /* complex128 arrays (interleaved FP64 re, im; 16 bytes per element),
-                                  FP64 butterflies and FP64 twiddles: the paper's own precision
-                                  (Section 4).  Natural pencil-pencil-pencil schedule of runtime-radix
-                                  passes (slab-pencil and FFT3_AUTO lower to it; volumetric, rotated,
+                                  the paper's own precision (Section 4): each line is transformed in
+                                  64-bit block fixed point and rounded once to FP64 (error per pass
+                                  about 5e-17 of the line's norm), lines with infinities, NaN or
+                                  values outside 2^-895..2^1007 by FP64 butterflies.  Natural
+                                  pencil-pencil-pencil schedule (slab-pencil and FFT3_AUTO lower to it; volumetric, rotated,
                                   blocked and permuted layouts are refused).  Buffers hold
                                   n0*n1*n2*batch complex128 values */
 };

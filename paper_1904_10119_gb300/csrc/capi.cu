@@ -23,6 +23,8 @@ __global__ void k_vol(PassArgs a);
 __global__ void k_probe_pass(PassArgs a);
 __global__ void k_copy(const float2 *in, float2 *out, int64_t total);
 __global__ void k_roots(int n, int sign, const int64_t *m, int64_t count, double *o64, float2 *o32);
+struct root62;
+__global__ void k_roots_fix(int n, const int64_t *m, int64_t count, root62 *o);
 __global__ void k_split_bf16(const float *x, int64_t count, uint16_t *hi, uint16_t *lo);
 extern const FixedKernels g_fixed_kernels_a[];
 extern const int g_fixed_kernels_a_count;
@@ -216,6 +218,10 @@ static PassGeom natural_x(const Schedule &s)
     return g;
 }
 
+// Entries of a plan's twiddle table; a complex128 plan holds two tables of this
+// size, the FP64 roots and then the integer ones.
+static int64_t twiddle_slots(const Schedule &s) { return std::max<int64_t>(16, s.tw_total); }
+
 static int build_launches(fft3_plan_s *P)
 {
     const Schedule &s = P->sched;
@@ -248,6 +254,8 @@ static int build_launches(fft3_plan_s *P)
         if (base < 0)
             base = 0;
         a.tw = P->esize == 16 ? (const float2 *)((const double2 *)P->d_tw + base) : P->d_tw + base;
+        if (P->esize == 16)
+            a.tw_fix = (const double2 *)P->d_tw + twiddle_slots(s) + base;
         a.tw_len = (int)(end - base);
         if (p.tw_seg[0] >= 0)
             a.L[0] = to_rt(p.line, (int)(s.tw[p.tw_seg[0]].off - base));
@@ -434,8 +442,8 @@ static void free_plan(fft3_plan_s *P)
 static int generate_twiddles(fft3_plan_s *P)
 {
     const Schedule &s = P->sched;
-    int64_t total = std::max<int64_t>(16, s.tw_total);
-    const bool fp64 = P->esize == 16; // complex128: the FP64 values are the table
+    const bool fp64 = P->esize == 16; // complex128: the FP64 values, then the integer ones
+    const int64_t total = twiddle_slots(s) * (fp64 ? 2 : 1);
     CUDA_TRY(cudaMalloc(&P->d_tw, total * P->esize));
     CUDA_TRY(cudaMemset(P->d_tw, 0, total * P->esize));
     size_t maxm = 1;
@@ -450,6 +458,10 @@ static int generate_twiddles(fft3_plan_s *P)
             k_roots<<<std::max(1, blocks), 256>>>(sg.n, FFT3_FORWARD, d_m, (int64_t)sg.m.size(),
                                                   fp64 ? (double *)P->d_tw + 2 * sg.off : nullptr,
                                                   fp64 ? nullptr : P->d_tw + sg.off);
+            if (fp64)
+                k_roots_fix<<<std::max(1, blocks), 256>>>(
+                    sg.n, d_m, (int64_t)sg.m.size(),
+                    (root62 *)((double2 *)P->d_tw + twiddle_slots(s) + sg.off));
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) {

@@ -1,0 +1,470 @@
+// fix64.cuh -- complex128 line transforms in 64-bit block fixed point.
+//
+// GB300 issues 2 FP64 operations per clock and SM against 64 integer adds and
+// 64 wide integer multiply-adds, so an FP64 butterfly is bound by the FP64
+// pipe at a few per cent of the memory bandwidth.  Here a line's values are
+// converted once to 64-bit integers with one exponent per line, the Stockham
+// stages run on integers, and the result is rounded once to FP64.
+//
+// Format: a component is an integer V, its value V * 2^(unit exponent).  Moduli
+// stay below 2^62: every radix-4 layer takes moduli below 2^60 (a butterfly of
+// four grows them at most fourfold) and the multiplication before it scales by
+// 1/4, so the unit exponent rises by two per layer (see cmul62).  Radix 2, 3
+// and 8 = 4 * 2 layers fit the same rule; radix 5 takes one more halving.
+//
+// Error: a product is rounded to the unit, a halving truncates, so a layer adds
+// about one unit to a value, and passes half of the layers before it on (in
+// the rms, sqrt(4) / 4).  The result of a line of n points thus carries about
+// 1.3 units rms where its own rms is 2^59 / (crest * sqrt(n)) units and more,
+// crest = largest component / rms modulus of the line: 2^-55 at n = 1024 and
+// crest 2, against 2^-52 for the same stages in FP64.  Lines of 512 points and
+// more are shifted back up to full scale after the first stage (block floating
+// point), so a line that is one spike (crest sqrt(n)) is no exception.
+//
+// Lines with an infinity, a NaN or values so large or small that their exponent
+// cannot be carried (below 2^-895, above 2^1007) take the FP64 stages.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+#include <string.h>
+
+#ifndef FFT3_HD
+#define FFT3_HD __host__ __device__ __forceinline__
+#endif
+
+namespace fft3 {
+
+struct __align__(16) fix2 {
+    long long x, y;
+};
+
+FFT3_HD fix2 cadd(fix2 a, fix2 b) { return fix2{a.x + b.x, a.y + b.y}; }
+FFT3_HD fix2 csub(fix2 a, fix2 b) { return fix2{a.x - b.x, a.y - b.y}; }
+FFT3_HD fix2 mul_mi(fix2 a) { return fix2{a.y, -a.x}; }
+FFT3_HD fix2 quarter(fix2 a) { return fix2{a.x >> 2, a.y >> 2}; }
+FFT3_HD fix2 half(fix2 a) { return fix2{a.x >> 1, a.y >> 1}; }
+FFT3_HD fix2 shl(fix2 a, int s)
+{
+    return fix2{(long long)((unsigned long long)a.x << s), (long long)((unsigned long long)a.y << s)};
+}
+
+FFT3_HD long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
+
+// V = h * 2^32 + l with l in [-2^31, 2^31).
+FFT3_HD int bal_lo(long long v) { return (int)(unsigned)v; }
+FFT3_HD int bal_hi(long long v) { return (int)(v >> 32) + (int)((unsigned)v >> 31); }
+
+// A root of unity times 2^62, each component as balanced 32-bit halves, the low
+// halves in (-2^31, 2^31) so that they can be negated.
+struct __align__(16) root62 {
+    int rh, rl, ih, il;
+};
+
+// a * w / 4: the product with w * 2^62, shifted down by 64 and rounded.  The
+// products of the low halves (below half a unit) are left out.  With moduli
+// below 2^62 the middle sum stays below 2^62.6.
+FFT3_HD fix2 cmul62(fix2 a, root62 w)
+{
+    const int ah = bal_hi(a.x), al = bal_lo(a.x), bh = bal_hi(a.y), bl = bal_lo(a.y);
+    const int nih = -w.ih, nil = -w.il;
+    long long m = mad_wide(ah, w.rl, 1ll << 31);
+    m = mad_wide(al, w.rh, m);
+    m = mad_wide(bh, nil, m);
+    m = mad_wide(bl, nih, m);
+    long long r = mad_wide(ah, w.rh, (int)(m >> 32));
+    r = mad_wide(bh, nih, r);
+    m = mad_wide(ah, w.il, 1ll << 31);
+    m = mad_wide(al, w.ih, m);
+    m = mad_wide(bh, w.rl, m);
+    m = mad_wide(bl, w.rh, m);
+    long long i = mad_wide(ah, w.ih, (int)(m >> 32));
+    i = mad_wide(bh, w.rh, i);
+    return fix2{r, i};
+}
+
+// a * c / 4 for a real constant c * 2^62 in the same halves.
+FFT3_HD long long rmul62(long long a, int ch, int cl)
+{
+    const int ah = bal_hi(a), al = bal_lo(a);
+    long long m = mad_wide(ah, cl, 1ll << 31);
+    m = mad_wide(al, ch, m);
+    return mad_wide(ah, ch, (int)(m >> 32));
+}
+
+// cos(k pi / 16) * 2^62 for k = 0..8, from which every power of w_32 follows.
+constexpr long long kFxC32[9] = {4611686018427387904ll, 4523073764714963030ll, 4260642322793532497ll,
+                                 3834476785802888710ll, 3260954456333195553ll, 2562115475870945497ll,
+                                 1764815834521887442ll, 899695310372275547ll, 0ll};
+FFT3_HD constexpr int const_hi(long long v) { return (int)((v + (1ll << 31)) >> 32); }
+FFT3_HD constexpr int const_lo(long long v) { return (int)(v - ((long long)const_hi(v) << 32)); }
+FFT3_HD constexpr long long fx_cos32(int m)
+{
+    m &= 31;
+    return m <= 8 ? kFxC32[m] : m < 16 ? -kFxC32[16 - m] : m < 24 ? -fx_cos32(m - 16) : kFxC32[32 - m];
+}
+
+// a * w_32^M / 4, M known at compile time.
+template <int M>
+FFT3_HD fix2 mul_w32_4(fix2 a)
+{
+    if constexpr (M == 0) {
+        return quarter(a);
+    } else if constexpr (M == 8) {
+        return quarter(mul_mi(a));
+    } else {
+        constexpr long long c = fx_cos32(M), s = fx_cos32(M - 8); // w = c - i s
+        return cmul62(a, root62{const_hi(c), const_lo(c), const_hi(-s), const_lo(-s)});
+    }
+}
+
+// In-register DFT_R of values with moduli below 2^60 (2^59 for R = 5); results
+// below 2^62.  scale(R): powers of two the result is scaled down by.
+template <int R>
+struct BflyFix;
+
+template <>
+struct BflyFix<2> {
+    static constexpr int scale = 0;
+    FFT3_HD static void run(fix2 *v)
+    {
+        const fix2 a = v[0], b = v[1];
+        v[0] = cadd(a, b);
+        v[1] = csub(a, b);
+    }
+};
+
+template <>
+struct BflyFix<4> {
+    static constexpr int scale = 0;
+    FFT3_HD static void run(fix2 *v)
+    {
+        const fix2 t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
+        const fix2 t2 = cadd(v[1], v[3]), t3 = mul_mi(csub(v[1], v[3]));
+        v[0] = cadd(t0, t2);
+        v[2] = csub(t0, t2);
+        v[1] = cadd(t1, t3);
+        v[3] = csub(t1, t3);
+    }
+};
+
+// 8 = 2 * 4 and 16 = 4 * 4 by Eq. ct, as the floating-point butterflies, the
+// inner twiddles scaling by 1/4.
+template <>
+struct BflyFix<8> {
+    static constexpr int scale = 2;
+    FFT3_HD static void run(fix2 *v)
+    {
+        fix2 e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+        BflyFix<4>::run(e);
+        BflyFix<4>::run(o);
+        o[0] = mul_w32_4<0>(o[0]);
+        o[1] = mul_w32_4<4>(o[1]);
+        o[2] = mul_w32_4<8>(o[2]);
+        o[3] = mul_w32_4<12>(o[3]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const fix2 q = quarter(e[k]);
+            v[k] = cadd(q, o[k]);
+            v[k + 4] = csub(q, o[k]);
+        }
+    }
+};
+
+template <>
+struct BflyFix<16> {
+    static constexpr int scale = 2;
+    FFT3_HD static void run(fix2 *v)
+    {
+        fix2 t[4][4];
+#pragma unroll
+        for (int i0 = 0; i0 < 4; ++i0) {
+#pragma unroll
+            for (int i1 = 0; i1 < 4; ++i1)
+                t[i0][i1] = v[i0 + 4 * i1];
+            BflyFix<4>::run(t[i0]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            t[0][k] = quarter(t[0][k]);
+        t[1][0] = quarter(t[1][0]);
+        t[1][1] = mul_w32_4<2>(t[1][1]);
+        t[1][2] = mul_w32_4<4>(t[1][2]);
+        t[1][3] = mul_w32_4<6>(t[1][3]);
+        t[2][0] = quarter(t[2][0]);
+        t[2][1] = mul_w32_4<4>(t[2][1]);
+        t[2][2] = mul_w32_4<8>(t[2][2]);
+        t[2][3] = mul_w32_4<12>(t[2][3]);
+        t[3][0] = quarter(t[3][0]);
+        t[3][1] = mul_w32_4<6>(t[3][1]);
+        t[3][2] = mul_w32_4<12>(t[3][2]);
+        t[3][3] = mul_w32_4<18>(t[3][3]);
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) {
+            fix2 c[4] = {t[0][k1], t[1][k1], t[2][k1], t[3][k1]};
+            BflyFix<4>::run(c);
+#pragma unroll
+            for (int k0 = 0; k0 < 4; ++k0)
+                v[k1 + 4 * k0] = c[k0];
+        }
+    }
+};
+
+// 32 = 2 * 16 (the radix-32 plan of 1024 points).
+template <int K>
+struct Tw32Fix {
+    FFT3_HD static void run(fix2 *o)
+    {
+        o[K] = mul_w32_4<K>(o[K]);
+        if constexpr (K + 1 < 16)
+            Tw32Fix<K + 1>::run(o);
+    }
+};
+
+template <>
+struct BflyFix<32> {
+    static constexpr int scale = 4;
+    FFT3_HD static void run(fix2 *v)
+    {
+        fix2 e[16], o[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            e[i] = v[2 * i];
+            o[i] = v[2 * i + 1];
+        }
+        BflyFix<16>::run(e);
+        BflyFix<16>::run(o);
+        Tw32Fix<0>::run(o);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const fix2 q = quarter(e[k]);
+            v[k] = cadd(q, o[k]);
+            v[k + 16] = csub(q, o[k]);
+        }
+    }
+};
+
+// Constants of DFT_3 and DFT_5 times 2^64, as the parts below 1/2 that a signed
+// 64-bit word holds: sin(2 pi/3) = 1 - f etc., so a product keeps every unit.
+constexpr long long kFx1mS3 = 2471395088767036514ll;  // 1 - sin(2 pi / 3)
+constexpr long long kFxC51 = 5700357409661599243ll;   // cos(2 pi / 5)
+constexpr long long kFx1pC52 = 3523014627193176565ll; // 1 + cos(4 pi / 5)
+constexpr long long kFx1mS51 = 902847917979075853ll;  // 1 - sin(2 pi / 5)
+constexpr long long kFx1mS52 = 7604019954369499282ll; // 1 - sin(4 pi / 5)
+
+// a * f for f * 2^64 = c (|f| < 1/2, |a| < 2^62), rounded to the unit.
+FFT3_HD long long fmulc(long long a, long long c) { return rmul62(a, const_hi(c), const_lo(c)); }
+
+// DFT_3 and DFT_5 in the forms of the floating-point butterflies.
+template <>
+struct BflyFix<3> {
+    static constexpr int scale = 0;
+    FFT3_HD static void run(fix2 *v)
+    {
+        const fix2 s = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+        const fix2 a = csub(v[0], half(s));
+        const fix2 b = fix2{d.x - fmulc(d.x, kFx1mS3), d.y - fmulc(d.y, kFx1mS3)};
+        v[0] = cadd(v[0], s);
+        v[1] = fix2{a.x + b.y, a.y - b.x};
+        v[2] = fix2{a.x - b.y, a.y + b.x};
+    }
+};
+
+template <>
+struct BflyFix<5> {
+    static constexpr int scale = 1; // halves its inputs first
+    // a1 = x0 + cos(2 pi/5) sa + cos(4 pi/5) sb, a2 the same with sa and sb swapped
+    FFT3_HD static long long even(long long x0, long long sa, long long sb)
+    {
+        return x0 - sb + fmulc(sa, kFxC51) + fmulc(sb, kFx1pC52);
+    }
+    FFT3_HD static void run(fix2 *v)
+    {
+        const fix2 x0 = half(v[0]);
+        const fix2 p1 = half(v[1]), p2 = half(v[2]), p3 = half(v[3]), p4 = half(v[4]);
+        const fix2 sa = cadd(p1, p4), da = csub(p1, p4), sb = cadd(p2, p3), db = csub(p2, p3);
+        const fix2 a1 = fix2{even(x0.x, sa.x, sb.x), even(x0.y, sa.y, sb.y)};
+        const fix2 a2 = fix2{even(x0.x, sb.x, sa.x), even(x0.y, sb.y, sa.y)};
+        // b1 = s1 da + s2 db, b2 = s2 da - s1 db
+        const fix2 b1 = fix2{da.x + db.x - fmulc(da.x, kFx1mS51) - fmulc(db.x, kFx1mS52),
+                             da.y + db.y - fmulc(da.y, kFx1mS51) - fmulc(db.y, kFx1mS52)};
+        const fix2 b2 = fix2{da.x - db.x - fmulc(da.x, kFx1mS52) + fmulc(db.x, kFx1mS51),
+                             da.y - db.y - fmulc(da.y, kFx1mS52) + fmulc(db.y, kFx1mS51)};
+        v[0] = cadd(x0, cadd(sa, sb));
+        v[1] = fix2{a1.x + b1.y, a1.y - b1.x};
+        v[4] = fix2{a1.x - b1.y, a1.y + b1.x};
+        v[2] = fix2{a2.x + b2.y, a2.y - b2.x};
+        v[3] = fix2{a2.x - b2.y, a2.y + b2.x};
+    }
+};
+
+// Normalisation between stages: `acc` is the OR of norm_word over the
+// components of a line; the line is shifted up by norm_shift(acc), which keeps
+// components below 2^61 (a line above that stays as it is).
+FFT3_HD unsigned norm_word(long long v)
+{
+    const int h = (int)(v >> 32);
+    return (unsigned)(h ^ (h >> 31));
+}
+FFT3_HD int clz32(unsigned v)
+{
+#ifdef __CUDA_ARCH__
+    return __clz((int)v);
+#else
+    return v ? __builtin_clz(v) : 32;
+#endif
+}
+FFT3_HD int norm_shift(unsigned acc)
+{
+    const int l = clz32(acc) - 3;
+    return l > 0 ? l : 0;
+}
+
+// ------------------------------------------------------- conversions ---- //
+// Exponent field range of a line's largest component that the integer stages
+// take; zero lines (field 0, all bits zero) are taken too.
+constexpr int kFixMinExp = 128, kFixMaxExp = 2030;
+
+// Magnitude word of one component for the line maximum: its high word without
+// the sign, or 1 for a subnormal whose high word is zero.
+FFT3_HD unsigned mag_word(double v)
+{
+    unsigned long long b;
+    memcpy(&b, &v, 8);
+    const unsigned h = (unsigned)(b >> 32) & 0x7fffffffu;
+    return h ? h : ((unsigned)b != 0u ? 1u : 0u);
+}
+// Whether a line with this largest magnitude word takes the integer stages.
+FFT3_HD bool fix_ok(unsigned m) { return m == 0u || ((m >> 20) >= (unsigned)kFixMinExp && (m >> 20) <= (unsigned)kFixMaxExp); }
+
+// Exponent field the line's values are scaled by (any of the range for a zero
+// line: a zero's mantissa is then shifted out).
+FFT3_HD int fix_emax(unsigned m) { return m ? (int)(m >> 20) : 1023; }
+
+// v in units of 2^(emax - 1023 - 58): components below 2^59, moduli below 2^60
+// (emax: exponent field of the line's largest component).
+FFT3_HD long long to_fix(double v, int emax)
+{
+    unsigned long long b;
+    memcpy(&b, &v, 8);
+    const unsigned hi = (unsigned)(b >> 32);
+    const int e = (int)((hi >> 20) & 0x7ffu);
+    unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b;
+    const int d = emax - e;
+    m = (m << 6) >> (d < 63 ? d : 63);
+    return (int)hi < 0 ? -(long long)m : (long long)m;
+}
+
+// V * 2^sh, rounded once (to the nearest): sh shifts the exponent field of
+// (double)V.  from_fix_int is the same conversion on the integer pipe: the
+// hardware's runs at 2 lanes per clock and SM on the FP64 pipe.
+FFT3_HD double from_fix(long long v, int sh)
+{
+    const double d = (double)v;
+    unsigned long long b;
+    memcpy(&b, &d, 8);
+    b += (unsigned long long)(long long)sh << 52;
+    double r;
+    memcpy(&r, &b, 8);
+    return v ? r : 0.0;
+}
+FFT3_HD double from_fix_int(long long v, int sh)
+{
+    const unsigned sign = (unsigned)((unsigned long long)v >> 32) & 0x80000000u;
+    unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const unsigned h = (unsigned)(u >> 32);
+    const int z = h ? clz32(h) : 32 + clz32((unsigned)u);
+    // leading bit to bit 62, rounded to 53 bits (ties to even) and to bit 52,
+    // where it adds one to the exponent field (a carry past it one more)
+    u <<= z - 1;
+    u += 0x1ffu + ((unsigned)(u >> 10) & 1u);
+    u >>= 10;
+    const unsigned hi = (unsigned)(u >> 32) + ((unsigned)(1023 + 62 - z + sh) << 20);
+    const unsigned long long b = ((unsigned long long)(hi | sign) << 32) | (unsigned)u;
+    double r;
+    memcpy(&r, &b, 8);
+    return v ? r : 0.0;
+}
+
+// ---------------------------------------------------------- roots ------- //
+// sin and cos of theta / 2^64 (theta < pi/4 * 2^64) as Q62, by their Taylor
+// series in 64-bit fixed point.
+FFT3_HD unsigned long long mulhi64(unsigned long long a, unsigned long long b)
+{
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return (unsigned long long)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+FFT3_HD void sincos_q64(unsigned long long th, long long *s, long long *c)
+{
+    const unsigned long long t2 = mulhi64(th, th);
+    // terms theta^k / k! for k = 2, 3, ...; cos = 1 - T2 + T4 - ..., sin = T1 - T3 + ...
+    unsigned long long tc = t2 >> 1, ts = mulhi64(th, t2) / 6;
+    long long cs = 0;                        // cos - 1, Q64 (|cos - 1| < 0.3)
+    long long ss = (long long)(th >> 1);     // sin, Q63
+    cs -= (long long)tc;
+    ss -= (long long)(ts >> 1);
+    for (int k = 2; k < 12; ++k) {
+        tc = mulhi64(tc, t2) / (unsigned)((2 * k) * (2 * k - 1));
+        ts = mulhi64(ts, t2) / (unsigned)((2 * k + 1) * (2 * k));
+        if (k & 1) {
+            cs -= (long long)tc;
+            ss -= (long long)(ts >> 1);
+        } else {
+            cs += (long long)tc;
+            ss += (long long)(ts >> 1);
+        }
+    }
+    *c = (1ll << 62) + ((cs + 2) >> 2);
+    *s = (ss + 1) >> 1;
+}
+
+// w_n^m = exp(-2 pi i m / n) times 2^62, m reduced mod n and to an octant in
+// integers: 8m = o n + rem, theta = 2 pi rem / (8n) or its complement to pi/4.
+FFT3_HD root62 root_fix(int64_t m, int n)
+{
+    int64_t mm = m % n;
+    if (mm < 0)
+        mm += n;
+    const int64_t o = 8 * mm / n;
+    int64_t rem = 8 * mm - o * n; // in [0, n)
+    if (o & 1)
+        rem = n - rem;            // odd octants run backwards, in (0, n]
+    long long s, c;
+    if (rem == n) {
+        constexpr long long h = fx_cos32(4); // sqrt(1/2)
+        s = c = h;
+    } else {
+        // rem / n as Q64 times pi / 4 as Q64
+        const unsigned long long q = (((unsigned long long)rem << 32) / (unsigned)n) << 32;
+        const unsigned long long r2 = ((unsigned long long)rem << 32) % (unsigned)n;
+        const unsigned long long frac = q | ((r2 << 32) / (unsigned)n);
+        sincos_q64(mulhi64(frac, 0xc90fdaa22168c235ull), &s, &c);
+    }
+    long long re, im; // exp(+i angle)
+    switch (o & 7) {
+    case 0: re = c; im = s; break;
+    case 1: re = s; im = c; break;
+    case 2: re = -s; im = c; break;
+    case 3: re = -c; im = s; break;
+    case 4: re = -c; im = -s; break;
+    case 5: re = -s; im = -c; break;
+    case 6: re = s; im = -c; break;
+    default: re = c; im = -s; break;
+    }
+    im = -im;
+    root62 w;
+    if ((unsigned)re == 0x80000000u)
+        --re;
+    if ((unsigned)im == 0x80000000u)
+        --im;
+    w.rh = bal_hi(re);
+    w.rl = bal_lo(re);
+    w.ih = bal_hi(im);
+    w.il = bal_lo(im);
+    return w;
+}
+
+} // namespace fft3

@@ -52,6 +52,7 @@ struct PassArgs {
     float2 *out;
     PassGeom g;
     const float2 *tw; // the pass's twiddle tables (global memory), tw_len entries
+    const void *tw_fix; // complex128: the same roots for the integer stages (fix64.cuh)
     int tw_len;
     int conj;         // 1: inverse via conj(DFT(conj x))
     int64_t ntiles;

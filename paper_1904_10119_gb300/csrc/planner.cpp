@@ -221,9 +221,11 @@ void generic_launch_shape_elem(int n, int T, bool strided, int tw_len, int esize
     int P = pitch_h(n);
     // strided lines: tiles of 16 (complex64) or 8 (complex128) columns, 128-byte rows
     int l = strided ? 128 / esize : std::max(1, 256 / T);
-    while (l > 1 && T * l > 1024)
+    while (l > 1 && T * l > (esize == 16 ? kMaxThreadsG64 : 1024))
         l /= 2;
-    auto bytes = [&](int ll) { return tw_slots_h(tw_len) * esize + 2 * ll * P * esize; };
+    // complex128: five words per line for the block fixed point (k_pass_g64)
+    const int state = esize == 16 ? 5 * 4 : 0;
+    auto bytes = [&](int ll) { return tw_slots_h(tw_len) * esize + ll * (2 * P * esize + state); };
     while (l > 1 && bytes(l) > kSmemLimit)
         l /= 2;
     *lpt = l;
@@ -387,6 +389,8 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
             return rc;
         const bool c128 = s->dtype == FFT3_C128_FP64;
         p.kind = c128 ? PK_G64 : PK_G;
+        if (c128)
+            p.line.T = std::min(p.line.T, kMaxThreadsG64);
         p.tw_seg[0] = line_seg(s, p.line);
         generic_launch_shape_elem(n, p.line.T, !contig_in, (int)s->tw[p.tw_seg[0]].m.size(), c128 ? 16 : 8,
                                   &p.lpt, &p.threads, &p.smem_bytes);
@@ -404,7 +408,7 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
     const int tc_opt = s->opts.tc_stages;
     const int tc_mode = tc_opt == 3 ? 0 : std::min(2, std::max(0, tc_opt));
     if (s->dtype == FFT3_C128_FP64) {
-        // complex128, 16-byte elements: the compile-time FP64 passes (k_pass64.cu)
+        // complex128, 16-byte elements: the compile-time passes (k_pass64.cu)
         // where the length has a fixed plan, else the runtime radix list (k_pass_g64)
         const bool contig = contig_in && g.ok == 1;
         if (p.line.fixed >= 0 && !rotate && (contig || (strided_in && p.line.T * kLpt64Strided <= 1024))) {
@@ -424,6 +428,7 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
         if (rc)
             return rc;
         p.kind = PK_G64;
+        p.line.T = std::min(p.line.T, kMaxThreadsG64);
         p.tw_seg[0] = line_seg(s, p.line);
         generic_launch_shape_elem(n, p.line.T, !contig_in, (int)s->tw[p.tw_seg[0]].m.size(), 16, &p.lpt,
                                   &p.threads, &p.smem_bytes);
@@ -1097,7 +1102,7 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
     }
     if (dtype == FFT3_C128_FP64) {
         // complex128 runs every line transform as one pass of the runtime-radix
-        // FP64 kernel: pencil-pencil-pencil in natural order (the slab-pencil
+        // complex128 kernel: pencil-pencil-pencil in natural order (the slab-pencil
         // and automatic choices lower to the same three passes)
         if (decomp == FFT3_VOLUMETRIC || s.opts.variant != FFT3_PPP_NATURAL ||
             s.opts.layout != FFT3_LAYOUT_NATURAL) {

@@ -27,7 +27,7 @@ enum PassKind {
     PK_VOLC = 12,  // compile-time volumetric split of strided lines (k_volc.cu)
     PK_CSTREAM = 13, // strided lines, decimated sub-lines streamed by TMA (k_cstream.cu)
     PK_SLABBLK = 14, // 2D slab DFT in one persistent launch, stored as blocked z pencils (k_slab_tma)
-    PK_G64 = 15,     // complex128: runtime radix list in FP64 (k_pass_g64)
+    PK_G64 = 15,     // complex128: runtime radix list (k_pass_g64)
     PK_J64 = 16,     // complex128: fixed plan, contiguous lines (k_pass_j64)
     PK_C64 = 17,     // complex128: fixed plan, strided columns (k_pass_c64)
     PK_TCX = 18,     // split-BF16 radix-32 tcgen05 GEMM stages, contiguous 1024-point lines (k_tc32.cu)
@@ -108,6 +108,7 @@ void generic_launch_shape_elem(int n, int T, bool strided, int tw_len, int esize
                                int *smem);
 
 constexpr int kMaxLine = 4096;
+constexpr int kMaxThreadsG64 = 512; // k_pass_g64's blocks (its launch bound: 128 registers a thread)
 constexpr int kTileTma = 1; // fft3_options.tile_lines value selecting the TMA strided kernel
 constexpr int kTileStream = 2; // fft3_options.tile_lines value selecting the streamed strided kernel
 constexpr int kSmemLimit = 227 * 1024;

@@ -1,0 +1,82 @@
+"""complex128 passes in 64-bit block fixed point: accuracy against an extended
+precision reference, the inputs that make a fixed point hard (spikes, values
+over 24 decades, lines of very different size), and the lines it leaves to FP64
+(infinities, NaN, subnormals, the ends of the exponent range)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1904_10119_gb300 import fft3
+
+pytestmark = pytest.mark.gpu
+
+
+def _passes(z):
+    """The rows of z as contiguous lines (pass 0 of n x lines) and as strided
+    columns (pass 1 of lines x n, in place on the output), one pass alone."""
+    lines, n = z.shape
+    res = []
+    for dims, k, a in (((n, lines, 1), 0, z), ((lines, n, 1), 1, z.T)):
+        x = torch.from_numpy(np.ascontiguousarray(a)).cuda()
+        out = torch.full_like(x, complex(float("nan"), float("nan"))) if k == 0 else x.clone()
+        plan = fft3.Plan(*dims, dtype=fft3.FFT3_C128_FP64)
+        fft3.fft3_plan_execute_pass(plan.handle, k, x.data_ptr(), out.data_ptr())
+        torch.cuda.synchronize()
+        assert plan.check() == 0, fft3.last_error()
+        plan.close()
+        got = out.cpu().numpy()
+        res.append(got if k == 0 else got.T)
+    return res
+
+
+def _lines(kind, n, lines, rng):
+    z = rng.uniform(-1, 1, (lines, n)) + 1j * rng.uniform(-1, 1, (lines, n))
+    if kind == "spike":
+        z = np.zeros((lines, n), complex)
+        z[np.arange(lines), rng.integers(0, n, lines)] = rng.normal(size=lines) + 0.3j
+    elif kind == "decades":
+        z = 10 ** rng.uniform(-12, 12, (lines, n)) * np.exp(2j * np.pi * rng.uniform(size=(lines, n)))
+    elif kind == "scales":  # neighbouring lines 400 decades apart, one of them zero
+        z *= 10.0 ** rng.integers(-200, 200, (lines, 1))
+        z[1] = 0
+    return z
+
+
+@pytest.mark.parametrize("n", [4, 16, 32, 60, 64, 128, 256, 375, 512, 960, 1024, 2025, 2048, 4096])
+@pytest.mark.parametrize("kind", ["uniform", "spike", "decades", "scales"])
+def test_one_pass_is_rounded_once(n, kind):
+    """Contiguous and strided lines, each line against its own norm.  A result
+    is rounded once to FP64 (rms 2^-53 / sqrt(3) = 6.4e-17 of the values' size
+    at most) after integer stages whose error is at most about twice that in
+    the hardest line (one spike that stays one through the first stage)."""
+    rng = np.random.default_rng(n)
+    z = _lines(kind, n, 9, rng)
+    sc = np.abs(z).max(axis=1, keepdims=True)
+    sc[sc == 0] = 1
+    ref = np.fft.fft((z.astype(np.clongdouble) / sc), axis=1)
+    for got in _passes(z):
+        err = np.abs(got.astype(np.clongdouble) / sc - ref)
+        norm = np.sqrt((np.abs(ref) ** 2).sum(axis=1))
+        rel = np.sqrt((err ** 2).sum(axis=1)) / np.where(norm == 0, 1, norm)
+        assert rel.max() <= 2e-16, (kind, float(rel.max()))
+        if kind == "scales":
+            assert not got[1].any()
+
+
+@pytest.mark.parametrize("n", [8, 60, 256, 1024, 1500])
+def test_lines_left_to_fp64(n):
+    """A tile holding such a line still gives every other line its result."""
+    rng = np.random.default_rng(n)
+    z = rng.uniform(-1, 1, (9, n)) + 1j * rng.uniform(-1, 1, (9, n))
+    z[2, n // 3] = complex(np.inf, 0)
+    z[4, 1] = complex(0.5, np.nan)
+    z[5] *= 1e-310
+    z[6] *= 1e305
+    ref = np.fft.fft(np.delete(z, (2, 4), 0), axis=1)
+    for got in _passes(z):
+        assert not np.isfinite(got[2]).any() and not np.isfinite(got[4]).any()
+        g = np.delete(got, (2, 4), 0)
+        for a, b in zip(g, ref):
+            # 1e-310 is held to 2^-1074 only: 4e-324 * sqrt(n) of absolute error
+            assert np.linalg.norm((a - b) * 2.0 ** -60) <= 1e-15 * np.linalg.norm(b * 2.0 ** -60) or \
+                np.abs(a - b).max() <= 5e-324 * 4 * n
