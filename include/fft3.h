@@ -249,10 +249,11 @@ int fft3_plan_create_ex(fft3_plan *out, int n0, int n1, int n2, int batch, int d
  *   executor:  one persistent launch with its counter reset; work items of
  *              every problem's phases (runtime radix lists) in waves that keep
  *              a problem's intermediate in L2.
- * FFT3_AUTO with tuning == NULL on a batch of at least 4 Mi values takes the
- * slab executor when every length is one of its lengths and every slab fits
- * one item (n1 * (n0 | 1) <= 96 * 97), else the segmented passes when every
- * line length has a compiled plan; other batches take the executor.  With
+ * FFT3_AUTO with tuning == NULL takes the slab executor on a batch of at least
+ * 1.5 Mi values when every length is one of its lengths and every slab fits
+ * one item (n1 * (n0 | 1) <= 96 * 97), else, from 4 Mi values on, the segmented
+ * passes when every line length has a compiled plan; other batches take the
+ * executor.  With
  * tuning codes: FFT3_TUNE_SLABZ on every code asks for the slab executor,
  * decomposition field 3 on every code for the segmented passes, anything
  * else for the executor.

@@ -179,6 +179,12 @@ constexpr SlabZPlan kSlabZPlans[] = {FFT3_SLABZ_Z_PLANS(FFT3_SZ_ZPLAN)};
 // values on (every line length compiled in seg_plans.h).
 constexpr int64_t kSegMinElems = 1ll << 22;
 
+// and the slab executor, where the batch fits it, from this many on: one
+// launch whose waits overlap.  24 problems of 3.9 Mi values: 48 us against 113
+// us for the item executor and 86 us for the segmented passes; 16 problems of
+// 1.8 Mi: 35, 80 and 68 us.
+constexpr int64_t kSlabzMinElems = 3ll << 19;
+
 // The compiled kernels for lines of length n in the segmented mode (x lines:
 // contiguous; y and z lines: strided), in the
 // order the radix_order field of a tuning code selects them (field value
@@ -458,7 +464,7 @@ static int batch_plan_host(BatchState *b, int count, const int *dims, const int6
     int slabz = tuning ? 1 : 0;
     for (int i = 0; slabz && i < count; ++i)
         slabz = (tuning[i] & FFT3_TUNE_SLABZ) ? 1 : 0;
-    // FFT3_AUTO without tuning codes takes it from kSegMinElems values on
+    // FFT3_AUTO without tuning codes takes it from kSlabzMinElems values on
     // when every length has its line variants and every slab fits the room of
     // an item (three blocks per SM); otherwise the segmented rule below
     if (!tuning && decomposition == FFT3_AUTO) {
@@ -482,7 +488,7 @@ static int batch_plan_host(BatchState *b, int count, const int *dims, const int6
             fit = has(n0, false) && has(n1, false) && has(n2, true) && n1 * (n0 | 1) <= kSlabzRoom;
             values += (int64_t)n0 * n1 * n2;
         }
-        slabz = fit && values >= kSegMinElems ? 1 : 0;
+        slabz = fit && values >= kSlabzMinElems ? 1 : 0;
     }
     b->slabz = slabz;
     for (int i = 0; i < count; ++i) {
@@ -749,9 +755,19 @@ static int batch_plan_host(BatchState *b, int count, const int *dims, const int6
             exp_n.push_back(K.n);
         }
         if (b->slabz) {
+            // lengths of this batch among dimensions d0..d1
+            auto used = [&](int n, int d0, int d1) {
+                for (int i = 0; i < count; ++i)
+                    for (int d = d0; d <= d1; ++d)
+                        if (dims[3 * i + d] == n)
+                            return true;
+                return false;
+            };
             // the z-tile plans' stage twiddles
             for (int k = 0; k < (int)(sizeof(kSlabZPlans) / sizeof(kSlabZPlans[0])) && k < 16; ++k) {
                 const SlabZPlan &q = kSlabZPlans[k];
+                if (!used(q.n, 2, 2))
+                    continue;
                 LineChoice lc{};
                 lc.n = q.n;
                 lc.fixed = -1;
@@ -774,6 +790,8 @@ static int batch_plan_host(BatchState *b, int count, const int *dims, const int6
             const int wl[] = {FFT3_SLABZ_WARP_PLANS(FFT3_SZ_LEN)};
 #undef FFT3_SZ_LEN
             for (int k = 0; k < (int)(sizeof(wl) / sizeof(wl[0])); ++k) {
+                if (!used(wl[k], 0, 1))
+                    continue;
                 std::vector<int64_t> e(wl[k]);
                 for (int m = 0; m < wl[k]; ++m)
                     e[m] = m;
@@ -950,17 +968,23 @@ extern "C" int fft3_plan_create_many(fft3_plan *out, int count, const int *dims,
         return bail(fail(FFT3_ERR_CUDA, "uploading the batched plan failed"));
     P->d_err = b->d_err;
     {
-        size_t maxm = 1;
+        // every table's exponents in one upload
+        std::vector<int64_t> m;
         for (auto &e : exps)
-            maxm = std::max(maxm, e.size());
+            m.insert(m.end(), e.begin(), e.end());
         int64_t *d_m = nullptr;
-        if (cudaMalloc(&d_m, maxm * sizeof(int64_t)) != cudaSuccess)
+        if (cudaMalloc(&d_m, std::max<size_t>(1, m.size()) * sizeof(int64_t)) != cudaSuccess)
             return bail(fail(FFT3_ERR_OOM, "twiddle scratch allocation failed"));
+        if (cudaMemcpy(d_m, m.data(), m.size() * sizeof(int64_t), cudaMemcpyHostToDevice) != cudaSuccess) {
+            cudaFree(d_m);
+            return bail(fail(FFT3_ERR_CUDA, "uploading the batched plan failed"));
+        }
+        size_t at = 0;
         for (size_t i = 0; i < exps.size(); ++i) {
-            cudaMemcpy(d_m, exps[i].data(), exps[i].size() * sizeof(int64_t), cudaMemcpyHostToDevice);
             int blocks = (int)std::max<int64_t>(1, ((int64_t)exps[i].size() + 255) / 256);
-            k_roots<<<blocks, 256>>>(exp_n[i], FFT3_FORWARD, d_m, (int64_t)exps[i].size(), nullptr,
+            k_roots<<<blocks, 256>>>(exp_n[i], FFT3_FORWARD, d_m + at, (int64_t)exps[i].size(), nullptr,
                                      b->d_tw + segs[i].first);
+            at += exps[i].size();
         }
         cudaError_t e = cudaDeviceSynchronize();
         cudaFree(d_m);
