@@ -31,14 +31,17 @@ extern const int g_fixed_kernels_a_count;
 extern const FixedKernels g_fixed_kernels_b[];
 extern const int g_fixed_kernels_b_count;
 
-extern const MixedKernels g_mixed_kernels_a[], g_mixed_kernels_b[], g_mixed_kernels_c[], g_mixed_kernels_d[];
+extern const MixedKernels g_mixed_j_a[], g_mixed_j_b[], g_mixed_j_c[], g_mixed_j_d[];
+extern const MixedKernels g_mixed_c_a[], g_mixed_c_b[], g_mixed_c_c[], g_mixed_c_d[];
 
-const MixedKernels *mixed_kernels(int n)
+const void *mixed_kernel(int n, bool contiguous)
 {
-    for (const MixedKernels *t : {g_mixed_kernels_a, g_mixed_kernels_b, g_mixed_kernels_c, g_mixed_kernels_d})
+    const MixedKernels *parts[2][4] = {{g_mixed_c_a, g_mixed_c_b, g_mixed_c_c, g_mixed_c_d},
+                                       {g_mixed_j_a, g_mixed_j_b, g_mixed_j_c, g_mixed_j_d}};
+    for (const MixedKernels *t : parts[contiguous ? 1 : 0])
         for (; t->n; ++t)
             if (t->n == n)
-                return t;
+                return t->func;
     return nullptr;
 }
 
@@ -282,11 +285,9 @@ static int build_launches(fft3_plan_s *P)
             L.func = fk ? fk->ctma : nullptr;
             L.tma = true;
             break;
-        case PK_G: {
-            const MixedKernels *mk = p.mixed ? mixed_kernels(p.line.n) : nullptr;
-            L.func = !p.mixed ? (const void *)&k_pass_g : mk ? (p.mixed == 1 ? mk->j : mk->c) : nullptr;
+        case PK_G:
+            L.func = p.mixed ? mixed_kernel(p.line.n, p.mixed == 1) : (const void *)&k_pass_g;
             break;
-        }
         case PK_G64: L.func = (const void *)&k_pass_g64; break;
         case PK_J64:
         case PK_C64: {

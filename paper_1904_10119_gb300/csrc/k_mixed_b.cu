@@ -1,6 +1,7 @@
-// Mixed-radix line passes, part B of the plan list.
+// Mixed-radix line passes, part B of the plan lists.
 #include "k_mixed.cuh"
 
 namespace fft3 {
-extern const MixedKernels g_mixed_kernels_b[] = {FFT3_MIXED_PLANS_B(FFT3_MIXED_ROW){0, nullptr, nullptr}};
+extern const MixedKernels g_mixed_j_b[] = {FFT3_MIXED_J_B(FFT3_MIXED_ROW_J){0, nullptr}};
+extern const MixedKernels g_mixed_c_b[] = {FFT3_MIXED_C_B(FFT3_MIXED_ROW_C){0, nullptr}};
 } // namespace fft3

@@ -75,15 +75,20 @@ const CStreamKernel *cstream_meta(int *count)
     return g_cstream_meta;
 }
 
-#define FFT3_MIXED_META(N, T, ...) {N, T, {__VA_ARGS__}},
-static const MixedPlanMeta g_mixed_meta[] = {FFT3_MIXED_PLANS(FFT3_MIXED_META)};
-#undef FFT3_MIXED_META
+#define FFT3_MIXED_META_J(N, T, LPT, MB, SH, PITCH, ...) {N, T, LPT, PITCH, {__VA_ARGS__}},
+#define FFT3_MIXED_META_C(N, T, LPT, MB, ...) {N, T, LPT, N, {__VA_ARGS__}},
+static const MixedPlanMeta g_mixed_j[] = {FFT3_MIXED_J(FFT3_MIXED_META_J)};
+static const MixedPlanMeta g_mixed_c[] = {FFT3_MIXED_C(FFT3_MIXED_META_C)};
+#undef FFT3_MIXED_META_J
+#undef FFT3_MIXED_META_C
 
-static const MixedPlanMeta *mixed_plan(int n)
+static const MixedPlanMeta *mixed_plan(int n, bool contiguous)
 {
-    for (const MixedPlanMeta &m : g_mixed_meta)
-        if (m.n == n)
-            return &m;
+    for (const MixedPlanMeta *m = contiguous ? g_mixed_j : g_mixed_c,
+                             *e = contiguous ? std::end(g_mixed_j) : std::end(g_mixed_c);
+         m != e; ++m)
+        if (m->n == n)
+            return m;
     return nullptr;
 }
 
@@ -544,19 +549,22 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
     // lines of a mixed plan's length, contiguous on both sides or strided columns:
     // the compile-time passes (k_mixed.cuh) under the default radix order; the
     // rotated store and radix orders 1..3 keep the runtime lists
-    const MixedPlanMeta *mp = p.kind == PK_G && order == 0 && !rotate && g.oblk == 0 ? mixed_plan(n) : nullptr;
-    if (mp && ((contig_in && g.ok == 1) || strided_in)) {
-        p.mixed = contig_in && g.ok == 1 ? 1 : 2;
+    const bool contig = contig_in && g.ok == 1;
+    const MixedPlanMeta *mp = p.kind == PK_G && order == 0 && !rotate && g.oblk == 0 && (contig || strided_in)
+                                  ? mixed_plan(n, contig)
+                                  : nullptr;
+    if (mp) {
+        p.mixed = contig ? 1 : 2;
         p.line.T = mp->T;
         for (p.line.nst = 0; p.line.nst < 8 && mp->rad[p.line.nst] > 0; ++p.line.nst)
             p.line.rad[p.line.nst] = mp->rad[p.line.nst];
     }
     p.tw_seg[0] = line_seg(s, p.line);
     int tw_len = (int)s->tw[p.tw_seg[0]].m.size();
-    if (p.mixed) {
-        p.lpt = p.mixed == 1 ? lpt_j(p.line.T) : mixed_lpt_c(n, p.line.T);
+    if (mp) {
+        p.lpt = mp->lpt;
         p.threads = p.line.T * p.lpt;
-        p.smem_bytes = (tw_slots_h(tw_len) + p.lpt * (p.mixed == 1 ? pitch_h(n) : n)) * 8;
+        p.smem_bytes = (tw_slots_h(tw_len) + p.lpt * mp->pitch) * 8;
     } else if (p.kind == PK_G) {
         generic_launch_shape(n, p.line.T, !contig_in, tw_len, &p.lpt, &p.threads, &p.smem_bytes);
     } else if (p.kind == PK_J) {
