@@ -279,6 +279,21 @@ static PassGeom geom_rotate(int d, int64_t n0, int64_t n1, int64_t n2, int64_t b
     return g;
 }
 
+// Contiguous lines that follow each other without a gap over c, a and b on both
+// sides are one run of lines, so tiles do not end at every a: with 45 lines per
+// plane and 42 per tile, half of the tiles held 3.
+static void merge_lines(PassGeom *g)
+{
+    if (g->A > 1 && g->ia == g->C * g->ic && g->oa == g->C * g->oc) {
+        g->C *= g->A;
+        g->A = 1;
+    }
+    if (g->A == 1 && g->B > 1 && g->ib == g->C * g->ic && g->ob == g->C * g->oc) {
+        g->C *= g->B;
+        g->B = 1;
+    }
+}
+
 static void set_tiles(PassPlan *p)
 {
     p->tiles_c = (p->g.C + p->lpt - 1) / p->lpt;
@@ -421,6 +436,8 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
             p.tw_seg[0] = line_seg(s, p.line);
             const int twl = tw_slots_h((int)s->tw[p.tw_seg[0]].m.size());
             p.lpt = contig ? lpt_j(p.line.T) : kLpt64Strided;
+            if (contig && s->opts.slab_mode != 4)
+                merge_lines(&p.g);
             p.threads = p.line.T * p.lpt;
             p.smem_bytes = (twl + (contig ? p.lpt * pitch_h(n) : p.lpt * n)) * 16;
             if (p.smem_bytes <= kSmemLimit) {
@@ -565,10 +582,14 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
         p.lpt = mp->lpt;
         p.threads = p.line.T * p.lpt;
         p.smem_bytes = (tw_slots_h(tw_len) + p.lpt * mp->pitch) * 8;
+        if (contig && s->opts.slab_mode != 4) // slab_mode 4 cuts its passes into chunks of a
+            merge_lines(&p.g);
     } else if (p.kind == PK_G) {
         generic_launch_shape(n, p.line.T, !contig_in, tw_len, &p.lpt, &p.threads, &p.smem_bytes);
     } else if (p.kind == PK_J) {
         p.threads = p.line.T * p.lpt;
+        if (s->opts.slab_mode != 4)
+            merge_lines(&p.g);
         p.smem_bytes = tw_slots_h(tw_len) * 8 + p.lpt * pitch_h(n) * 8;
     } else if (p.kind == PK_JROT) {
         p.threads = p.line.T * p.lpt;
@@ -1125,12 +1146,12 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
             s.opts.variant = FFT3_PPP_BLOCKED;
     }
     if (decomp == FFT3_AUTO) {
-        // Fixed default when no cost model is loaded: slab-pencil when a whole
-        // slab fits one block's shared memory (one HBM sweep fewer), else
-        // pencil-pencil-pencil, whose strided passes stream their sub-lines
-        // (measured faster than the L2-resident slab kernel at 1024 x 1024).
-        int twl = 2 * tw_slots_h(n0) + 2 * tw_slots_h(n1);
-        decomp = slab_smem(n0, n1, twl) <= kSmemLimit ? FFT3_SLAB_PENCIL : FFT3_PENCIL3;
+        // Fixed default when no cost model is loaded: pencil-pencil-pencil, whose
+        // passes are compiled for every length, but slab-pencil for slabs of at most
+        // 256 values, where one launch less counts (16^3: 10.0 against 12.2 us;
+        // 30^3 x 10: 13.0 against 12.5; 96 x 96 x 1000: 211 against 87: the slab
+        // kernel runs runtime radix lists).
+        decomp = (int64_t)n0 * n1 <= 256 ? FFT3_SLAB_PENCIL : FFT3_PENCIL3;
         // and with the blocked intermediate when it applies and the natural z lines
         // would be at least 4 MiB apart (1024^3: 8.68 against 9.41 ms; at 512^3, 2 MiB
         // apart, the natural layout measured 1.053 against 1.067 ms)
