@@ -147,6 +147,8 @@ __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(
     float2 *res = smem + tw_slots(a.tw_len); // QP slots of M x LPT, slot s at s*M*LPT
     float2 *stg = res + QP * M * LPT;        // G*S staging buffers of M x LPT; group g owns g*S .. g*S+S-1
     load_twiddles(tw, a.tw, a.tw_len);
+    if constexpr (P == 1)
+        pdl_wait();
     const int tid = threadIdx.x, g = tid / GT, gtid = tid % GT;
     const int l = gtid % LPT, t1 = gtid / LPT;
     const bool conj = a.conj != 0;

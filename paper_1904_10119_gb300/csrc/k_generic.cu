@@ -60,6 +60,7 @@ __global__ void k_pass_g(PassArgs a)
     const int P = line_pitch(L.n);
     float2 *b0 = tw + tw_slots(a.tw_len), *b1 = b0 + a.lpt * P;
     load_twiddles(tw, a.tw, a.tw_len);
+    pdl_wait();
     for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
         __syncthreads();
         const TileG t = tile_g(a, tile);
@@ -182,6 +183,7 @@ __global__ void __launch_bounds__(512) k_pass_g64(PassArgs a) // kMaxThreadsG64
     const root62 *twg = reinterpret_cast<const root62 *>(a.tw_fix);
     for (int i = threadIdx.x; i < a.tw_len; i += blockDim.x)
         tw[i] = twg[i];
+    pdl_wait();
     int scale = 0; // powers of two the stages scale down by
     for (int s = 0; s < L.nst; ++s)
         scale += fix_scale_rt(L.rad[s]) + (s ? 2 : 0);
@@ -236,6 +238,7 @@ __global__ void k_slab(PassArgs a)
     float2 *b0 = smem + tw_slots(a.tw_len);
     float2 *b1 = b0 + n1 * P;
     load_twiddles(tw, a.tw, a.tw_len);
+    pdl_wait();
     const bool conj = a.conj != 0;
     const int nel = n0 * n1;
     for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {

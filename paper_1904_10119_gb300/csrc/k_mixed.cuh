@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(T *LPT, MB) k_mixed_j(PassArgs a)
     float2 *tw = smem;
     float2 *buf = smem + tw_slots(a.tw_len);
     load_twiddles(tw, a.tw, a.tw_len);
+    pdl_wait();
     const int t = threadIdx.x % T, l = threadIdx.x / T;
     const bool conj = a.conj != 0;
     for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
@@ -55,6 +56,7 @@ __global__ void __launch_bounds__(T *LPT, MB) k_mixed_c(PassArgs a)
     float2 *tw = smem;
     float2 *buf = smem + tw_slots(a.tw_len);
     load_twiddles(tw, a.tw, a.tw_len);
+    pdl_wait();
     const int l = threadIdx.x % LPT, t = threadIdx.x / LPT;
     const bool conj = a.conj != 0;
     for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {

@@ -253,6 +253,7 @@ __device__ __forceinline__ void pass64(const PassArgs &a)
     const root62 *twg = reinterpret_cast<const root62 *>(a.tw_fix);
     for (int i = threadIdx.x; i < a.tw_len; i += T * LPT)
         tw[i] = twg[i];
+    pdl_wait();
     const double2 *twd = reinterpret_cast<const double2 *>(a.tw);
     const double2 *in = reinterpret_cast<const double2 *>(a.in);
     double2 *out = reinterpret_cast<double2 *>(a.out);
