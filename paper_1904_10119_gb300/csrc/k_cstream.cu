@@ -147,8 +147,6 @@ __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(
     float2 *res = smem + tw_slots(a.tw_len); // QP slots of M x LPT, slot s at s*M*LPT
     float2 *stg = res + QP * M * LPT;        // G*S staging buffers of M x LPT; group g owns g*S .. g*S+S-1
     load_twiddles(tw, a.tw, a.tw_len);
-    if constexpr (P == 1)
-        pdl_wait();
     const int tid = threadIdx.x, g = tid / GT, gtid = tid % GT;
     const int l = gtid % LPT, t1 = gtid / LPT;
     const bool conj = a.conj != 0;
@@ -195,6 +193,9 @@ __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(
         }
     };
     if (gtid == 0) {
+        // only the loading threads wait for the passes before: all other accesses follow their loads
+        if constexpr (P == 1)
+            pdl_wait();
         for (int k = 0; k < S; ++k)
             issue(k);
     }
@@ -236,11 +237,11 @@ __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(
                     issue(k + S); // the staging buffer is read out: refill it
             } else {
                 // (I) first stage, radix R1, NS = 1: inputs x_q[t1 + r*T1] of column l
-                float2 x[R1];
+                pk2 x[R1];
 #pragma unroll
                 for (int r = 0; r < R1; ++r) {
                     const float2 e = sb[(t1 + r * T1) * LPT + l];
-                    x[r] = conj ? cconj(e) : e;
+                    x[r] = conj ? cconj(pk2(e)) : pk2(e);
                 }
                 if (group_sync_or<G, GT>(g, late) && !failed) {
                     failed = true;
@@ -269,7 +270,7 @@ __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(
                 continue;
             }
             // (I) second stage, radix R2, NS = R1, in place in slot q
-            float2 y[BPT2][R2];
+            pk2 y[BPT2][R2];
 #pragma unroll
             for (int bb = 0; bb < BPT2; ++bb) {
                 const int q2 = t1 + bb * T1;
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(
             const float2 *twf = tw + (M - 1);
 #pragma unroll 2
             for (int kk = r * MP + tf; kk < (r + 1) * MP; kk += TF) {
-                float2 z[Q];
+                pk2 z[Q];
 #pragma unroll
                 for (int s = 0; s < Q; ++s) {
                     const float2 *src = (s / QP == r) ? res : peer;

@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(256) k_segw(SegArgs a)
         const bool valid = c < (int64_t)cb.n1 * cb.n2;
         const float2 *ip = a.src + cb.off + (valid ? c * N : 0);
         float2 *op = a.out + cb.off + (valid ? c * N : 0);
-        float2 v[2][R];
+        pk2 v[2][R];
         WL::load(v, ip, u, valid, conj);
         WL::run(v, tw, u);
         WL::store(v, op, u, valid, conj);
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(256) k_segw_s(SegArgs a)
         const bool valid = c < lines;
         const float2 *ip = a.src + cb.off + (valid ? first : 0);
         float2 *op = a.out + cb.off + (valid ? first : 0);
-        float2 v[2][R];
+        pk2 v[2][R];
         WL::load_strided(v, ip, es, u, valid, conj);
         WL::run(v, tw, u);
         WL::store_strided(v, op, es, u, valid, conj);

@@ -76,7 +76,7 @@ __device__ __noinline__ void sz_rows_warp(const float2 *src, float2 *A, int pitc
     for (int r0 = 0; r0 < rows; r0 += RPR) {
         const int row = r0 + l;
         const bool valid = row < rows;
-        float2 v[2][R];
+        pk2 v[2][R];
         WL::load(v, src + (int64_t)(valid ? row : 0) * N, u, valid, conj);
         WL::run(v, tw, u);
         if (valid) {
@@ -110,7 +110,7 @@ __device__ __noinline__ void sz_cols_warp(float2 *A, int pitch, int cols, int w,
         const bool valid = c < cols;
         const int cs = valid ? c / w : 0, cc = valid ? c - cs * w : 0;
         float2 *p = A + cs * slab_stride + cc;
-        float2 v[2][R];
+        pk2 v[2][R];
         WL::load_strided(v, p, pitch, u, valid, false);
         WL::run(v, tw, u);
         WL::store_strided(v, p, pitch, u, valid, false);
@@ -162,7 +162,7 @@ __device__ __noinline__ void sz_ztiles(float2 *base, int64_t t0, int64_t t1, int
         SzGLoad src{p, es, valid, conj};
         GStore dst{p, es, valid, conj};
         SzTile<LPT> sm{buf + (g < G ? g : 0) * (LPT * N) + l, valid};
-        EngineFixed<N, T, 1, Rad>::template run<true, false>(t, src, sm, dst, tw);
+        EngineFixed<N, T, 1, Rad>::template run<true, false>(t, src, sm, dst, reinterpret_cast<const pk2 *>(tw));
     }
 }
 

@@ -62,7 +62,7 @@ struct WarpLine {
     // Strided lines (element j at p[j * es]): the lanes of a line sit on
     // different rows, adjacent lines (columns) in adjacent lane groups, so a
     // warp's access covers one run of adjacent columns per row.
-    __device__ __forceinline__ static void load_strided(float2 (&v)[2][R], const float2 *p, int64_t es, int u,
+    __device__ __forceinline__ static void load_strided(pk2 (&v)[2][R], const float2 *p, int64_t es, int u,
                                                         bool valid, bool conj)
     {
 #pragma unroll
@@ -70,12 +70,12 @@ struct WarpLine {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const float2 x = valid ? p[(int64_t)(2 * u + e + L * i) * es] : make_float2(0.f, 0.f);
-                v[e][i] = conj ? cconj(x) : x;
+                v[e][i] = conj ? cconj(pk2(x)) : pk2(x);
             }
         }
     }
 
-    __device__ __forceinline__ static void store_strided(float2 (&v)[2][R], float2 *p, int64_t es, int u,
+    __device__ __forceinline__ static void store_strided(pk2 (&v)[2][R], float2 *p, int64_t es, int u,
                                                          bool valid, bool conj)
     {
         if (!valid)
@@ -92,7 +92,7 @@ struct WarpLine {
     // v[e][i] = x[2u + e + L i] (conjugated for the inverse); zeros when !valid.
     // Streaming loads (evict first from L1): each value is read once, and L1
     // keeps what is read again (twiddle tables).
-    __device__ __forceinline__ static void load(float2 (&v)[2][R], const float2 *p, int u, bool valid, bool conj)
+    __device__ __forceinline__ static void load(pk2 (&v)[2][R], const float2 *p, int u, bool valid, bool conj)
     {
         if (valid && ((reinterpret_cast<uintptr_t>(p) & 15) == 0)) {
 #pragma unroll
@@ -117,7 +117,7 @@ struct WarpLine {
         }
     }
 
-    __device__ __forceinline__ static void run(float2 (&v)[2][R], const Tw &tw, int u)
+    __device__ __forceinline__ static void run(pk2 (&v)[2][R], const Tw &tw, int u)
     {
         // (I), (II)
 #pragma unroll
@@ -139,7 +139,7 @@ struct WarpLine {
                 for (int k = 0; k < R; ++k) {
                     const float px = __shfl_xor_sync(0xffffffffu, v[e][k].x, m);
                     const float py = __shfl_xor_sync(0xffffffffu, v[e][k].y, m);
-                    const float2 d = make_float2(fmaf(sg, v[e][k].x, px), fmaf(sg, v[e][k].y, py));
+                    const pk2 d(fmaf(sg, v[e][k].x, px), fmaf(sg, v[e][k].y, py));
                     v[e][k] = cmul(d, tw.net[s][e]);
                 }
             }
@@ -147,14 +147,14 @@ struct WarpLine {
         // (IV) last step, h = 1, in registers
 #pragma unroll
         for (int k = 0; k < R; ++k) {
-            const float2 a = v[0][k], b = v[1][k];
+            const pk2 a = v[0][k], b = v[1][k];
             v[0][k] = cadd(a, b);
             v[1][k] = csub(a, b);
         }
     }
 
     // X[k' + R rev(2u + e)] = v[e][k'] (conjugated for the inverse).
-    __device__ __forceinline__ static void store(float2 (&v)[2][R], float2 *p, int u, bool valid, bool conj)
+    __device__ __forceinline__ static void store(pk2 (&v)[2][R], float2 *p, int u, bool valid, bool conj)
     {
         if (!valid)
             return;
@@ -165,8 +165,8 @@ struct WarpLine {
                 if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
 #pragma unroll
                     for (int k = 0; k < R; k += 2) {
-                        const float2 a = conj ? cconj(v[e][k]) : v[e][k];
-                        const float2 b = conj ? cconj(v[e][k + 1]) : v[e][k + 1];
+                        const pk2 a = conj ? cconj(v[e][k]) : v[e][k];
+                        const pk2 b = conj ? cconj(v[e][k + 1]) : v[e][k + 1];
                         *reinterpret_cast<float4 *>(q + k) = make_float4(a.x, a.y, b.x, b.y);
                     }
                     continue;
