@@ -63,7 +63,15 @@
 // refilled as soon as they are read, then one radix-Q stage with twiddles
 // w_N^{q k'} stores the lines.  With P = 2 a cluster of two blocks shares a
 // tile of LPT = 32 columns, each block holding half of the sub-lines.  The
-// line's twiddle table is the stage-major table of (R1, R2, Q).
+// line's twiddle table is the stage-major table of (R1, R2, Q).  The pairs are
+// bound by the exchange (remote reads and two cluster barriers per tile), so
+// they want several blocks per SM: 512 points as 8 sub-lines of 8 x 8 (two
+// blocks) 239 us on 512 x 512 x 256, as 4 of 16 x 8 (one block) 291; 256 points
+// 76 us at 256^3, two groups against one 84, two sub-lines of 16 x 8 80; 128
+// points 68 us on 1024 x 128 x 128, two groups 102; 64 points 28 us on 1024 x
+// 64 x 64, four sub-lines of 4 x 4 29.  The compiled split over four blocks
+// (k_volc.cu) took 460 us for 256 points on 512 x 512 x 256, the runtime split
+// (k_vol.cu), which still takes the other lengths, 2.9 ms for 64 points on 0.5 GB.
 // Row: N, Q, R1, R2, G, S, LPT, P.
 #define FFT3_CSTREAM_LIST(X)             \
     X(1024, 4, 16, 16, 2, 1, 16, 1)      \
@@ -75,7 +83,11 @@
     X(512, 4, 16, 8, 2, 1, 16, 1)        \
     X(512, 2, 16, 16, 1, 2, 16, 1)       \
     X(512, 2, 16, 16, 2, 1, 16, 1)       \
-    X(512, 4, 16, 8, 2, 1, 32, 2)
+    X(512, 8, 8, 8, 2, 1, 32, 2)         \
+    X(512, 4, 16, 8, 2, 1, 32, 2)        \
+    X(256, 4, 8, 8, 2, 1, 32, 2)         \
+    X(128, 4, 8, 4, 1, 1, 32, 2)         \
+    X(64, 2, 8, 4, 1, 1, 32, 2)
 
 namespace fft3 {
 
