@@ -106,26 +106,14 @@ __device__ __forceinline__ void tile_sync()
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// Staging buffer as a tile accessor (line = column, position = row of the
-// sub-line), conjugating on load for the inverse transform.
-template <int LPT>
-struct StageTile {
-    const float2 *p;
-    bool conj;
-    __device__ __forceinline__ float2 operator()(int l, int j) const
-    {
-        const float2 v = p[j * LPT + l];
-        return conj ? cconj(v) : v;
-    }
-};
-
 // TC = 0: FP32 sub-line stages.  TC = 1: the first 16-point stage of every
 // sub-line on the tensor cores in split BF16 (tc_stage.cuh); TC = 2: both.
 template <int N, int Q, int R1, int R2, int G, int S, int LPT, int P, int TC>
 __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(N, Q, Q / P, LPT, G *S), G *LPT *R2))
     k_cstream(PassArgs a, const __grid_constant__ CUtensorMap tin)
 {
-    static_assert(TC == 0 || (R1 == 16 && R2 == 16 && P == 1), "tensor-core sub-lines are 16 x 16");
+    static_assert(TC == 0 || (R1 == 16 && R2 == 16 && P == 1 && LPT == 16),
+                  "tensor-core sub-lines are 16 x 16, in tiles of 16 columns");
     constexpr int M = R1 * R2;
     constexpr int T1 = M / R1;          // threads per column in a group (= first-stage butterflies)
     constexpr int GT = LPT * T1;        // threads per group
@@ -227,8 +215,7 @@ __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(
             float2 *slot = res + q * M * LPT;
             if constexpr (TC > 0) {
                 // (I) first 16-point stage on the tensor cores: staging buffer -> slot q
-                tc_stage16<M, 1, LPT, true>(StageTile<LPT>{sb, conj}, TileColSmem<LPT>{slot}, tw, wtc,
-                                            gtid >> 5, GT / 32);
+                tc_stage16_cols16<M, 1>(sb, slot, conj, tw, wtc, gtid >> 5, GT / 32);
                 if (group_sync_or<G, GT>(g, late) && !failed) {
                     failed = true;
                     k_fail = k;
@@ -265,8 +252,7 @@ __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(
                 // (I) second 16-point stage on the tensor cores, in place in slot q: with
                 // NS = 16 and M = 256 the outputs of a butterfly are its own inputs'
                 // positions, and a warp reads all its inputs before its MMAs
-                tc_stage16<M, R1, LPT, true>(TileColSmem<LPT>{slot}, TileColSmem<LPT>{slot}, tw + (R1 - 1), wtc,
-                                             gtid >> 5, GT / 32);
+                tc_stage16_cols16<M, R1>(slot, slot, false, tw + (R1 - 1), wtc, gtid >> 5, GT / 32);
                 continue;
             }
             // (I) second stage, radix R2, NS = R1, in place in slot q

@@ -81,8 +81,8 @@
     X(1024, 8, 16, 8, 2, 2, 16, 1)       \
     X(1024, 8, 8, 16, 2, 2, 16, 1)       \
     X(512, 4, 16, 8, 2, 1, 16, 1)        \
-    X(512, 2, 16, 16, 1, 2, 16, 1)       \
     X(512, 2, 16, 16, 2, 1, 16, 1)       \
+    X(512, 2, 16, 16, 1, 2, 16, 1)       \
     X(512, 8, 8, 8, 2, 1, 32, 2)         \
     X(512, 4, 16, 8, 2, 1, 32, 2)        \
     X(256, 4, 8, 8, 2, 1, 32, 2)         \

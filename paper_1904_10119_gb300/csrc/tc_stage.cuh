@@ -35,11 +35,9 @@ __device__ __forceinline__ uint32_t bf16x2_bits(__nv_bfloat16 lo, __nv_bfloat16 
 // (x0, x1) -> packed high parts and packed low parts.
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t &hi, uint32_t &lo)
 {
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
-    const __nv_bfloat16 l0 = __float2bfloat16_rn(x0 - __bfloat162float(h0));
-    const __nv_bfloat16 l1 = __float2bfloat16_rn(x1 - __bfloat162float(h1));
-    hi = bf16x2_bits(h0, h1);
-    lo = bf16x2_bits(l0, l1);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(x1), "f"(x0));
+    const float l0 = x0 - __uint_as_float(hi << 16), l1 = x1 - __uint_as_float(hi & 0xffff0000u);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(l1), "f"(l0));
 }
 
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
@@ -147,6 +145,71 @@ __device__ __forceinline__ void tc_stage16(const Src &src, const Dst &dst, const
             tc_butterfly<NB, LPT, GROUP_LINES>(grp, 2 * t + (e & 1), ol, oq);
             const int base = (NS == 1) ? oq * 16 : (oq / NS) * NS * 16 + (oq % NS);
             dst(ol, base + k * NS, make_float2(d[0][e], d[1][e]));
+        }
+    }
+}
+
+// The same stage on a position-major tile of 16 columns (value of position j,
+// column c at p[j * 16 + c]), a warp taking the 16 butterflies of one q at a
+// time.  A lane reads two adjacent columns, 2g and 2g + 1, of its four inputs r
+// with 16-byte loads, so a warp's load covers whole 128-byte rows (the eight
+// columns of one MMA alone put its four rows on the same banks: two wavefronts
+// for one); the even columns form one MMA's N side, the odd ones another's, and
+// their outputs land as four adjacent columns 4t .. 4t + 3 per lane, stored with
+// 16-byte stores (the two halves in opposite order in odd rows, so that eight
+// lanes cover all banks).  `src` and `dst` may be the same tile where a
+// butterfly's outputs take its inputs' places (NS * 16 == N): a warp has read
+// its inputs when its products run.
+template <int N, int NS>
+__device__ __forceinline__ void tc_stage16_cols16(const float2 *src, float2 *dst, bool conj, const float2 *tw,
+                                                  const TcW &w, int warp, int nwarps)
+{
+    constexpr int NB = N / 16;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const float sg = conj ? -1.f : 1.f;
+    for (int q = warp; q < NB; q += nwarps) {
+        float2 v[2][4]; // [column 2g + h][input]
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int r = 2 * t + (e & 1) + ((e & 2) ? 8 : 0);
+            const float4 x = *reinterpret_cast<const float4 *>(src + (q + r * NB) * 16 + 2 * g);
+            v[0][e] = make_float2(x.x, sg * x.y);
+            v[1][e] = make_float2(x.z, sg * x.w);
+            if constexpr (NS > 1) {
+                if (r > 0) {
+                    const float2 c = tw[(r - 1) * NS + (q % NS)];
+                    v[0][e] = cmul(v[0][e], c);
+                    v[1][e] = cmul(v[1][e], c);
+                }
+            }
+        }
+        float d[2][2][4] = {}; // [h][yr | yi][fragment]
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t bh[2][2], bl[2][2]; // [xr|xi][register]
+            split_pair(v[h][0].x, v[h][1].x, bh[0][0], bl[0][0]);
+            split_pair(v[h][2].x, v[h][3].x, bh[0][1], bl[0][1]);
+            split_pair(v[h][0].y, v[h][1].y, bh[1][0], bl[1][0]);
+            split_pair(v[h][2].y, v[h][3].y, bh[1][1], bl[1][1]);
+#pragma unroll
+            for (int mb = 0; mb < 2; ++mb)
+#pragma unroll
+                for (int kb = 0; kb < 2; ++kb) {
+                    mma_bf16_16816(d[h][mb], w.lo[mb][kb], bh[kb][0], bh[kb][1]);
+                    mma_bf16_16816(d[h][mb], w.hi[mb][kb], bl[kb][0], bl[kb][1]);
+                    mma_bf16_16816(d[h][mb], w.hi[mb][kb], bh[kb][0], bh[kb][1]);
+                }
+        }
+        const int base = (NS == 1) ? q * 16 : (q / NS) * NS * 16 + (q % NS);
+#pragma unroll
+        for (int k8 = 0; k8 < 2; ++k8) {
+            float4 *o = reinterpret_cast<float4 *>(dst + (base + (g + 8 * k8) * NS) * 16 + 4 * t);
+            const float4 lo = make_float4(d[0][0][2 * k8], d[0][1][2 * k8], d[1][0][2 * k8], d[1][1][2 * k8]);
+            const float4 hi = make_float4(d[0][0][2 * k8 + 1], d[0][1][2 * k8 + 1], d[1][0][2 * k8 + 1],
+                                          d[1][1][2 * k8 + 1]);
+            const bool odd = g & 1;
+            o[odd ? 1 : 0] = odd ? hi : lo;
+            o[odd ? 0 : 1] = odd ? lo : hi;
         }
     }
 }
