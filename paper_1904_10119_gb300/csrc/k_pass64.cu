@@ -17,7 +17,7 @@
 //
 // What bounds it: latency at 16 warps per SM (128 registers: 16 values of four
 // words each) and the integer pipe, 48% busy; the FP64 pipe carries only half of
-// the final roundings.  256^3: 594 us, 2.7 TB/s per pass, against 2502 us with
+// the final roundings.  256^3: 572 us, 2.8 TB/s per pass, against 2502 us with
 // FP64 stages (2 lanes per clock and SM).  Tried: radix-8 plans (24 warps, one
 // exchange more) 671 us; up to 168 registers (12 warps) 630 us.
 // The runtime-radix kernel (k_pass_g64) covers the other lengths.
@@ -242,44 +242,47 @@ struct FixTile<N, T, Radices<R, Rest...>, SEG> {
     }
 };
 
-// The tile loop of both kernels; LINES: contiguous lines, else columns.
-template <int N, int T, class Rad, int LPT, bool LINES>
+// The tile loop of both kernels; LINES: contiguous lines, else columns, G tiles
+// side by side in a block (one barrier domain).
+template <int N, int T, class Rad, int LPT, int G, bool LINES>
 __device__ __forceinline__ void pass64(const PassArgs &a)
 {
-    constexpr int S = line_pitch(N);
-    __shared__ unsigned slots[2][2][LPT]; // [tile parity][largest magnitude word, normalisation word][line]
+    constexpr int S = line_pitch(N), GT = T * LPT, NT = GT * G;
+    __shared__ unsigned slots[2][2][G * LPT]; // [tile parity][largest magnitude word, normalisation word][line]
     root62 *tw = reinterpret_cast<root62 *>(smem64());
     unsigned char *buf = smem64() + (size_t)tw_slots(a.tw_len) * 16;
     const root62 *twg = reinterpret_cast<const root62 *>(a.tw_fix);
-    for (int i = threadIdx.x; i < a.tw_len; i += T * LPT)
+    for (int i = threadIdx.x; i < a.tw_len; i += NT)
         tw[i] = twg[i];
     pdl_wait();
     const double2 *twd = reinterpret_cast<const double2 *>(a.tw);
     const double2 *in = reinterpret_cast<const double2 *>(a.in);
     double2 *out = reinterpret_cast<double2 *>(a.out);
-    const int t = LINES ? threadIdx.x % T : threadIdx.x / LPT;
-    const int l = LINES ? threadIdx.x / T : threadIdx.x % LPT;
+    const int g = G > 1 ? threadIdx.x / GT : 0, gt = G > 1 ? threadIdx.x % GT : threadIdx.x;
+    const int t = LINES ? gt % T : gt / LPT;
+    const int l = LINES ? gt / T : gt % LPT;
     // lanes of a line that are adjacent in a warp (whole warps only)
-    constexpr int SEG = LINES && (T * LPT) % 32 == 0 && (T & (T - 1)) == 0 ? (T < 32 ? T : 32) : 1;
+    constexpr int SEG = LINES && NT % 32 == 0 && (T & (T - 1)) == 0 ? (T < 32 ? T : 32) : 1;
     const bool conj = a.conj != 0;
     int par = 0;
-    for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x, par ^= 1) {
-        for (int i = threadIdx.x; i < 2 * LPT; i += T * LPT)
-            slots[par][i / LPT][i % LPT] = 0;
+    for (int64_t tile0 = (int64_t)blockIdx.x * G; tile0 < a.ntiles; tile0 += (int64_t)gridDim.x * G, par ^= 1) {
+        for (int i = threadIdx.x; i < 2 * G * LPT; i += NT)
+            slots[par][i / (G * LPT)][i % (G * LPT)] = 0;
         __syncthreads();
-        const TileId id = decode_tile(tile, a.tiles_c, a.g.A, LPT);
+        const bool live = G == 1 || tile0 + g < a.ntiles;
+        const TileId id = decode_tile(live ? tile0 + g : tile0, a.tiles_c, a.g.A, LPT);
         const int64_t c = id.c0 + l;
-        const bool valid = c < a.g.C;
+        const bool valid = live && c < a.g.C;
         const G64Load src{in + c * a.g.ic + id.a * a.g.ia + id.b * a.g.ib, LINES ? 1 : a.g.ij, valid, conj};
         const G64Store dst{out + c * a.g.oc + id.a * a.g.oa + id.b * a.g.ob, LINES ? 1 : a.g.ok, valid, conj};
-        unsigned *mx = &slots[par][0][l], *nrm = &slots[par][1][l];
+        unsigned *mx = &slots[par][0][g * LPT + l], *nrm = &slots[par][1][g * LPT + l];
         if constexpr (LINES) {
             const Smem64Line<fix2> sm{reinterpret_cast<fix2 *>(buf) + l * S};
             const Smem64Line<double2> smd{reinterpret_cast<double2 *>(buf) + l * S};
             FixTile<N, T, Rad, SEG>::run(t, src, sm, smd, dst, tw, twd, mx, nrm);
         } else {
-            const Smem64Col<fix2, LPT> sm{reinterpret_cast<fix2 *>(buf) + l};
-            const Smem64Col<double2, LPT> smd{reinterpret_cast<double2 *>(buf) + l};
+            const Smem64Col<fix2, LPT> sm{reinterpret_cast<fix2 *>(buf) + g * (LPT * N) + l};
+            const Smem64Col<double2, LPT> smd{reinterpret_cast<double2 *>(buf) + g * (LPT * N) + l};
             FixTile<N, T, Rad, SEG>::run(t, src, sm, smd, dst, tw, twd, mx, nrm);
         }
     }
@@ -289,22 +292,25 @@ __device__ __forceinline__ void pass64(const PassArgs &a)
 constexpr int fix_min_blocks(int threads) { return threads >= 512 ? 1 : 512 / threads; }
 
 template <int N, int T, class Rad, int LPT>
-__global__ void __launch_bounds__(T *LPT, fix_min_blocks(T * LPT)) k_pass_j64(PassArgs a) { pass64<N, T, Rad, LPT, true>(a); }
+__global__ void __launch_bounds__(T *LPT, fix_min_blocks(T * LPT)) k_pass_j64(PassArgs a) { pass64<N, T, Rad, LPT, 1, true>(a); }
 
-template <int N, int T, class Rad, int LPT>
-__global__ void __launch_bounds__(T *LPT, fix_min_blocks(T * LPT)) k_pass_c64(PassArgs a) { pass64<N, T, Rad, LPT, false>(a); }
+template <int N, int T, class Rad, int LPT, int G>
+__global__ void __launch_bounds__(T *LPT *G, fix_min_blocks(T *LPT *G)) k_pass_c64(PassArgs a)
+{
+    pass64<N, T, Rad, LPT, G, false>(a);
+}
 
 template <int N, int T, class Rad>
 constexpr const void *pass_c64_ptr()
 {
     if constexpr (T * kLpt64Strided <= 1024)
-        return (const void *)&k_pass_c64<N, T, Rad, kLpt64Strided>;
+        return (const void *)&k_pass_c64<N, T, Rad, kLpt64Strided, groups64(T)>;
     else
         return nullptr;
 }
 
 #define FFT3_KERNEL64_ROW(ID, N, T, ...)                                                              \
-    {ID, (const void *)&k_pass_j64<N, T, Radices<__VA_ARGS__>, lpt_j(T)>,                            \
+    {ID, (const void *)&k_pass_j64<N, T, Radices<__VA_ARGS__>, lpt_j64(T)>,                           \
      pass_c64_ptr<N, T, Radices<__VA_ARGS__>>()},
 
 static const Fixed64Kernels g_fixed64[] = {FFT3_FIXED_PLANS_A(FFT3_KERNEL64_ROW)

@@ -435,11 +435,12 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
             p.kind = contig ? PK_J64 : PK_C64;
             p.tw_seg[0] = line_seg(s, p.line);
             const int twl = tw_slots_h((int)s->tw[p.tw_seg[0]].m.size());
-            p.lpt = contig ? lpt_j(p.line.T) : kLpt64Strided;
+            p.lpt = contig ? lpt_j64(p.line.T) : kLpt64Strided;
             if (contig && s->opts.slab_mode != 4)
                 merge_lines(&p.g);
-            p.threads = p.line.T * p.lpt;
-            p.smem_bytes = (twl + (contig ? p.lpt * pitch_h(n) : p.lpt * n)) * 16;
+            const int groups = contig ? 1 : groups64(p.line.T);
+            p.threads = p.line.T * p.lpt * groups;
+            p.smem_bytes = (twl + (contig ? p.lpt * pitch_h(n) : groups * p.lpt * n)) * 16;
             if (p.smem_bytes <= kSmemLimit) {
                 set_tiles(&p);
                 *out = p;
