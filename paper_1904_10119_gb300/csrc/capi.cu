@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "capi_internal.h"
+#include "mixed64_plans.h"
 #include "mixed_plans.h"
 #include "roots.cuh"
 
@@ -42,6 +43,17 @@ const void *mixed_kernel(int n, bool contiguous)
         for (; t->n; ++t)
             if (t->n == n)
                 return t->func;
+    return nullptr;
+}
+
+extern const Mixed64Kernels g_mixed64_a[], g_mixed64_b[], g_mixed64_c[], g_mixed64_d[], g_mixed64_e[], g_mixed64_f[];
+
+const Mixed64Kernels *mixed64_kernels(int n)
+{
+    for (const Mixed64Kernels *t : {g_mixed64_a, g_mixed64_b, g_mixed64_c, g_mixed64_d, g_mixed64_e, g_mixed64_f})
+        for (; t->n; ++t)
+            if (t->n == n)
+                return t;
     return nullptr;
 }
 
@@ -302,7 +314,11 @@ static int build_launches(fft3_plan_s *P)
         case PK_G:
             L.func = p.mixed ? mixed_kernel(p.line.n, p.mixed == 1) : (const void *)&k_pass_g;
             break;
-        case PK_G64: L.func = (const void *)&k_pass_g64; break;
+        case PK_G64: {
+            const Mixed64Kernels *mk = p.mixed ? mixed64_kernels(p.line.n) : nullptr;
+            L.func = !p.mixed ? (const void *)&k_pass_g64 : mk ? (p.mixed == 1 ? mk->j : mk->c) : nullptr;
+            break;
+        }
         case PK_J64:
         case PK_C64: {
             const Fixed64Kernels *k64 = p.line.fixed >= 0 ? fixed64_kernels(p.line.fixed) : nullptr;

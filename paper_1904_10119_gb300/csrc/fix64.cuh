@@ -298,6 +298,106 @@ struct BflyFix<5> {
     }
 };
 
+// cos and sin of 2 pi m / N times 2^62 for m <= N/2: the inner twiddles of the
+// composite butterflies.
+constexpr long long kFxCos9[5] = {
+    4611686018427387904ll, 3532756447825785444ll, 800810873071977681ll, -2305843009213693952ll,
+    -4333567320897763126ll};
+constexpr long long kFxSin9[5] = {
+    0ll, 2964334632409774423ll, 4541624145405292212ll, 3993837246235628775ll,
+    1577289512995517789ll};
+constexpr long long kFxCos10[6] = {
+    4611686018427387904ll, 3730932361629093763ll, 1425089352415399811ll, -1425089352415399811ll,
+    -3730932361629093763ll, -4611686018427387904ll};
+constexpr long long kFxSin10[6] = {
+    0ll, 2710681029835013083ll, 4385974038932618941ll, 4385974038932618941ll,
+    2710681029835013083ll, 0ll};
+constexpr long long kFxCos12[7] = {
+    4611686018427387904ll, 3993837246235628775ll, 2305843009213693952ll, 0ll,
+    -2305843009213693952ll, -3993837246235628775ll, -4611686018427387904ll};
+constexpr long long kFxSin12[7] = {
+    0ll, 2305843009213693952ll, 3993837246235628775ll, 4611686018427387904ll,
+    3993837246235628775ll, 2305843009213693952ll, 0ll};
+constexpr long long kFxCos15[8] = {
+    4611686018427387904ll, 4212984814208232069ll, 3085820261846986643ll, 1425089352415399811ll,
+    -482052452579138307ll, -2305843009213693952ll, -3730932361629093763ll, -4510909614262386453ll};
+constexpr long long kFxSin15[8] = {
+    0ll, 1875741690054758654ll, 3427150601320760278ll, 4385974038932618941ll,
+    4586422719889771737ll, 3993837246235628775ll, 2710681029835013083ll, 958823437611858663ll};
+template <int N>
+FFT3_HD constexpr long long fx_cos_n(int m)
+{
+    const int k = m <= N / 2 ? m : N - m;
+    return N == 9 ? kFxCos9[k < 5 ? k : 0] : N == 10 ? kFxCos10[k < 6 ? k : 0] : N == 12 ? kFxCos12[k < 7 ? k : 0]
+         : kFxCos15[k < 8 ? k : 0];
+}
+template <int N>
+FFT3_HD constexpr long long fx_sin_n(int m)
+{
+    const int k = m <= N / 2 ? m : N - m;
+    const long long v = N == 9 ? kFxSin9[k < 5 ? k : 0] : N == 10 ? kFxSin10[k < 6 ? k : 0]
+                      : N == 12 ? kFxSin12[k < 7 ? k : 0] : kFxSin15[k < 8 ? k : 0];
+    return m <= N / 2 ? v : -v;
+}
+
+// DFT_{A B} by Eq. ct (DFT_B, inner twiddles w_{AB}^{i0 k1} / 4, DFT_A); NT is
+// the table the twiddles come from (AB or a multiple).
+template <int A, int B, int NT, int I>
+struct CtFixTw {
+    FFT3_HD static void run(fix2 (*t)[B])
+    {
+        if constexpr (I < A * B) {
+            constexpr int m = (I / B) * (I % B) * (NT / (A * B)) % NT;
+            fix2 &v = t[I / B][I % B];
+            if constexpr (m == 0) {
+                v = quarter(v);
+            } else {
+                constexpr long long c = fx_cos_n<NT>(m), s = fx_sin_n<NT>(m);
+                v = cmul62(v, root62{const_hi(c), const_lo(c), const_hi(-s), const_lo(-s)});
+            }
+            CtFixTw<A, B, NT, I + 1>::run(t);
+        }
+    }
+};
+
+template <int A, int B, int NT>
+struct BflyFixCt {
+    static constexpr int scale = BflyFix<B>::scale + 2 + BflyFix<A>::scale;
+    FFT3_HD static void run(fix2 *v)
+    {
+        fix2 t[A][B];
+#pragma unroll
+        for (int i0 = 0; i0 < A; ++i0) {
+#pragma unroll
+            for (int i1 = 0; i1 < B; ++i1)
+                t[i0][i1] = v[i0 + A * i1];
+            BflyFix<B>::run(t[i0]);
+        }
+        CtFixTw<A, B, NT, 0>::run(t);
+#pragma unroll
+        for (int k1 = 0; k1 < B; ++k1) {
+            fix2 c[A];
+#pragma unroll
+            for (int i0 = 0; i0 < A; ++i0)
+                c[i0] = t[i0][k1];
+            BflyFix<A>::run(c);
+#pragma unroll
+            for (int k0 = 0; k0 < A; ++k0)
+                v[k1 + B * k0] = c[k0];
+        }
+    }
+};
+template <>
+struct BflyFix<6> : BflyFixCt<2, 3, 12> {};
+template <>
+struct BflyFix<9> : BflyFixCt<3, 3, 9> {};
+template <>
+struct BflyFix<10> : BflyFixCt<2, 5, 10> {};
+template <>
+struct BflyFix<12> : BflyFixCt<4, 3, 12> {};
+template <>
+struct BflyFix<15> : BflyFixCt<3, 5, 15> {};
+
 // Normalisation between stages: `acc` is the OR of norm_word over the
 // components of a line; the line is shifted up by norm_shift(acc), which keeps
 // components below 2^61 (a line above that stays as it is).

@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <sstream>
 
+#include "mixed64_plans.h"
 #include "mixed_plans.h"
 #include "plans.h"
 #include "roots.cuh"
@@ -90,6 +91,28 @@ static const MixedPlanMeta *mixed_plan(int n, bool contiguous)
         if (m->n == n)
             return m;
     return nullptr;
+}
+
+#define FFT3_MIXED64_META(N, T, LPT, SH, PITCH, ...) {N, T, LPT, PITCH, {__VA_ARGS__}},
+static const Mixed64Meta g_mixed64[] = {FFT3_MIXED64(FFT3_MIXED64_META)};
+#undef FFT3_MIXED64_META
+
+static const Mixed64Meta *mixed64_plan(int n)
+{
+    for (const Mixed64Meta &m : g_mixed64)
+        if (m.n == n)
+            return &m;
+    return nullptr;
+}
+
+// A mixed plan's threads and radix list as the pass's line.
+template <class Meta>
+static void set_mixed_line(LineChoice *lc, const Meta &m)
+{
+    lc->fixed = -1;
+    lc->T = m.T;
+    for (lc->nst = 0; lc->nst < 8 && m.rad[lc->nst] > 0; ++lc->nst)
+        lc->rad[lc->nst] = m.rad[lc->nst];
 }
 
 int fixed_plan_count() { return g_nmeta; }
@@ -428,8 +451,8 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
     const int tc_opt = s->opts.tc_stages;
     const int tc_mode = tc_opt == 3 ? 0 : std::min(2, std::max(0, tc_opt));
     if (s->dtype == FFT3_C128_FP64) {
-        // complex128, 16-byte elements: the compile-time passes (k_pass64.cu)
-        // where the length has a fixed plan, else the runtime radix list (k_pass_g64)
+        // complex128, 16-byte elements: the compile-time passes (k_pass64.cuh)
+        // where the length has a fixed or mixed plan, else the runtime radix list (k_pass_g64)
         const bool contig = contig_in && g.ok == 1;
         if (p.line.fixed >= 0 && !rotate && (contig || (strided_in && p.line.T * kLpt64Strided <= 1024))) {
             p.kind = contig ? PK_J64 : PK_C64;
@@ -446,6 +469,23 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
                 *out = p;
                 return FFT3_OK;
             }
+        }
+        const Mixed64Meta *mp = order == 0 && !rotate && g.oblk == 0 && (contig || strided_in) ? mixed64_plan(n) : nullptr;
+        if (mp) {
+            p.kind = PK_G64;
+            p.mixed = contig ? 1 : 2;
+            set_mixed_line(&p.line, *mp);
+            p.tw_seg[0] = line_seg(s, p.line);
+            const int twl = tw_slots_h((int)s->tw[p.tw_seg[0]].m.size());
+            const int groups = contig ? 1 : groups64(mp->T);
+            p.lpt = contig ? mp->lpt : kLpt64Strided;
+            p.threads = mp->T * p.lpt * groups;
+            p.smem_bytes = (twl + (contig ? p.lpt * mp->pitch : groups * p.lpt * n)) * 16;
+            if (contig && s->opts.slab_mode != 4)
+                merge_lines(&p.g);
+            set_tiles(&p);
+            *out = p;
+            return FFT3_OK;
         }
         rc = choose_line(n, order, false, &p.line, err);
         if (rc)
@@ -573,9 +613,7 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
                                   : nullptr;
     if (mp) {
         p.mixed = contig ? 1 : 2;
-        p.line.T = mp->T;
-        for (p.line.nst = 0; p.line.nst < 8 && mp->rad[p.line.nst] > 0; ++p.line.nst)
-            p.line.rad[p.line.nst] = mp->rad[p.line.nst];
+        set_mixed_line(&p.line, *mp);
     }
     p.tw_seg[0] = line_seg(s, p.line);
     int tw_len = (int)s->tw[p.tw_seg[0]].m.size();

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1904_10119_gb300 import fft3
+from paper_1904_10119_gb300 import fft3, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -61,6 +61,22 @@ def test_one_pass_is_rounded_once(n, kind):
         assert rel.max() <= 2e-16, (kind, float(rel.max()))
         if kind == "scales":
             assert not got[1].any()
+
+
+@pytest.mark.parametrize("n", [n for n in synth.smooth_sizes(3, 512) if n & (n - 1)])
+def test_mixed_plans_are_rounded_once(n):
+    """Every mixed-radix plan (contiguous and strided), on values over 24 decades:
+    the bound of the test above."""
+    z = _lines("decades", n, 9, np.random.default_rng(n))
+    sc = np.abs(z).max(axis=1, keepdims=True)
+    ref = np.fft.fft(z.astype(np.clongdouble) / sc, axis=1)
+    for k, dims in ((0, (n, 9, 1)), (1, (9, n, 1))):
+        p = fft3.fft3_plan_schedule(*dims, 1, fft3.FFT3_C128_FP64)["passes"][k]
+        assert p.get("compiled") and p["line"]["n"] == n
+    for got in _passes(z):
+        err = np.abs(got.astype(np.clongdouble) / sc - ref)
+        rel = np.sqrt((err ** 2).sum(axis=1) / (np.abs(ref) ** 2).sum(axis=1))
+        assert rel.max() <= 2e-16, float(rel.max())
 
 
 @pytest.mark.parametrize("n", [8, 60, 256, 1024, 1500])
