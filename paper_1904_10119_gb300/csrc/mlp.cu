@@ -45,7 +45,7 @@ __device__ __forceinline__ float gelu_grad_f(float x)
 // Loss and gradient of a minibatch in one launch, for the widths the model is
 // used at (H = 32, 64 or 128, F <= 64): the layer-by-layer kernels below took
 // nine launches of 2 to 10 us each (16 steps of 128 samples, F = 32, H = 64:
-// 1339 us; with this kernel 267 us, most of it launches and the copies of the
+// 1335 us; with this kernel 220 us, a third of it launches and the copies of the
 // parameters).  What bounds it: latency, a minibatch being a few microseconds of
 // work for a handful of SMs.
 // A cluster of 8 blocks holds a copy of the parameters each and takes chunks of
@@ -54,7 +54,7 @@ __device__ __forceinline__ float gelu_grad_f(float x)
 // pass, and only h1, dz1, dz2 and the inputs go through shared memory, for the
 // weight gradients, whose sums over all chunks stay in registers.  At the end
 // every block sums its share of the parameters over the cluster's shared
-// memories.  More than 512 samples are spread over several clusters whose sums a
+// memories.  More than 128 samples are spread over several clusters whose sums a
 // second kernel adds.  All sums run in a fixed order.
 constexpr int kGradCluster = 8, kGradChunk = 16, kGradThreads = 256, kGradMaxF = 64, kGradMaxClusters = 16;
 
@@ -84,10 +84,18 @@ __global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThre
           *b3 = w3 + H, *red = b3 + 4, *grad = red + 8 * (3 * H + 2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     asm volatile("griddepcontrol.wait;" ::: "memory"); // the Adam step before may still run
-    for (int i = tid; i < H * F; i += kGradThreads)
-        w1[(i / F) * FP + i % F] = p[L.w1 + i];
-    for (int i = tid; i < H * H; i += kGradThreads)
-        w2[(i / H) * (H + 1) + i % H] = p[L.w2 + i];
+    // a warp copies rows n = warp, warp + 8, ... (every load of a row set in flight at once)
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+        const int n = warp + 8 * i;
+#pragma unroll
+        for (int j = 0; j < J; ++j)
+            w2[n * (H + 1) + lane + 32 * j] = p[L.w2 + n * H + lane + 32 * j];
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (lane + 32 * j < F)
+                w1[n * FP + lane + 32 * j] = p[L.w1 + n * F + lane + 32 * j];
+    }
     for (int i = tid; i < H; i += kGradThreads) {
         b1[i] = p[L.b1 + i];
         b2[i] = p[L.b2 + i];
@@ -100,9 +108,12 @@ __global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThre
     const int chunks = (B + kGradChunk - 1) / kGradChunk;
     for (int c = blockIdx.x; c < chunks; c += gridDim.x) {
         __syncthreads(); // parameters loaded, or the previous chunk's sums done
-        for (int i = tid; i < kGradChunk * XP; i += kGradThreads) {
-            const int b = c * kGradChunk + i / XP, k = i % XP;
-            xs[i] = b < B && k < F ? X[(int64_t)(idx ? idx[b] : b) * F + k] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int r = 2 * warp + q, b = c * kGradChunk + r;
+            const int64_t row = b < B ? (int64_t)(idx ? idx[b] : b) * F : 0;
+            for (int k = lane; k < XP; k += 32)
+                xs[r * XP + k] = b < B && k < F ? X[row + k] : 0.f;
         }
         __syncthreads();
         // forward: samples s0 and s0 + 1, units lane + 32 j
@@ -111,6 +122,7 @@ __global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThre
 #pragma unroll
         for (int j = 0; j < J; ++j)
             z1[0][j] = z1[1][j] = b1[lane + 32 * j];
+#pragma unroll 8
         for (int k = 0; k < F; ++k) {
             const float x0 = xs[s0 * XP + k], x1 = xs[(s0 + 1) * XP + k];
 #pragma unroll
@@ -189,6 +201,7 @@ __global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThre
             }
         __syncthreads();
         // weight gradients over the chunk's samples
+#pragma unroll 4
         for (int s = 0; s < kGradChunk; ++s) {
             float hv[J], xv[2];
 #pragma unroll
@@ -488,9 +501,9 @@ static int mlp_gradient(fft3_mlp_s *m, const float *X, const float *y, const int
 {
     const MlpLayout &L = m->L;
     const void *f = grad_fused_kernel(L);
-    // chunks of one cluster's blocks up to 512 samples, then two chunks per block
+    // a chunk per block while the clusters last (a chunk takes 5 us, the second kernel 3)
     const int chunks = (B + kGradChunk - 1) / kGradChunk;
-    int clusters = chunks <= 4 * kGradCluster ? 1 : std::min(kGradMaxClusters, (chunks + 15) / 16);
+    int clusters = std::min(kGradMaxClusters, (chunks + kGradCluster - 1) / kGradCluster);
     float *g0 = clusters > 1 ? m->grad_ws : m->d_g;
     const float *p = m->d_p;
     float *loss0 = m->loss;
