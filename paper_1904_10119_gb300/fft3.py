@@ -194,7 +194,10 @@ def _flat(dims):
 
 
 def fft3_plan_execute(plan: int, in_ptr: int, out_ptr: int, stream: int = 0) -> None:
-    _check(load().fft3_plan_execute(_P(plan), _P(in_ptr), _P(out_ptr), _P(stream)))
+    # plain integers: ctypes converts them to the declared void pointers
+    rc = (_lib or load()).fft3_plan_execute(plan, in_ptr, out_ptr, stream)
+    if rc < 0:
+        _check(rc)
 
 
 FFT3_NOALLOC_MAX_ELEMENTS = 1 << 21
@@ -399,8 +402,10 @@ class Plan:
         want = torch.complex128 if self.dtype == FFT3_C128_FP64 else torch.complex64
         assert x.is_cuda and out.is_cuda and x.dtype == want and out.dtype == want
         assert x.is_contiguous() and out.is_contiguous()
-        s = stream if stream is not None else torch.cuda.current_stream()
-        fft3_plan_execute(self.handle, x.data_ptr(), out.data_ptr(), s.cuda_stream)
+        # the current stream's handle without a Stream object around it: a transform of
+        # a few microseconds is bound by this call
+        s = stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        fft3_plan_execute(self.handle, x.data_ptr(), out.data_ptr(), s)
 
     def describe(self) -> dict:
         return fft3_plan_describe(self.handle)
