@@ -420,10 +420,17 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
     p.src = src;
     p.dst = dst;
     int order = s->opts.radix_order;
-    int rc = choose_line(n, order, true, &p.line, err);
+    const bool contig_in = g.ij == 1;
+    // Contiguous complex64 lines of 16, 64 and 128 points take their second candidate
+    // first (4 x 4, 8 x 8, 8 x 16): more threads per line make longer runs of each load
+    // and store.  134 MB: 16 points 63 against 176 us, 64 points 49 against 62, 128
+    // points 49 against 53 (as strided columns the first candidates lead).
+    const bool swap = s->dtype != FFT3_C128_FP64 && contig_in && g.ok == 1 && !rotate && order >= 0 &&
+                      (n == 16 || n == 64 || n == 128);
+    const int cands = swap ? (int)fixed_candidates(n).size() : 1;
+    int rc = choose_line(n, swap && order % cands < 2 ? 1 - order % cands : order, true, &p.line, err);
     if (rc)
         return rc;
-    const bool contig_in = g.ij == 1;
     const bool strided_in = g.ic == 1 && g.oc == 1;
     if (g.ijb > 0 || g.okb > 0) {
         // lines in runs over exchange blocks: the runtime-radix kernels
