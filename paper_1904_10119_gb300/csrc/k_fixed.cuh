@@ -76,7 +76,7 @@ constexpr const void *pass_c_tc_ptr()
 
 #define FFT3_KERNEL_ROW(ID, N, T, ...)                                                          \
     {ID,                                                                                        \
-     (const void *)&fft3::k_pass_j<N, T, fft3::Radices<__VA_ARGS__>, fft3::lpt_j(T), false>,    \
+     (const void *)&fft3::k_pass_j<N, T, fft3::Radices<__VA_ARGS__>, fft3::lpt_jl(T), false>,   \
      (const void *)&fft3::k_pass_j<N, T, fft3::Radices<__VA_ARGS__>, fft3::lpt_rot(T), true>,   \
      fft3::pass_c_ptr<N, T, fft3::Radices<__VA_ARGS__>, fft3::lpt_c(T, 16)>(),                  \
      fft3::pass_c_ptr<N, T, fft3::Radices<__VA_ARGS__>, fft3::lpt_c(T, 8)>(),                   \

@@ -589,7 +589,7 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
         p.lpt = lpt_rot(p.line.T);
     } else if (p.line.fixed >= 0 && !rotate && contig_in && g.ok == 1 && n > 1) {
         p.kind = PK_J;
-        p.lpt = lpt_j(p.line.T);
+        p.lpt = lpt_jl(p.line.T);
     } else if (!rotate && strided_in && n > 1 && (s->opts.tile_lines == 0 || s->opts.tile_lines == kTileStream) &&
                cstream_pick(n, order, g, 1) >= 0) {
         set_cstream(&p, cstream_pick(n, order, g, 1));

@@ -201,6 +201,9 @@ constexpr int slab_tma_smem(int n, int lpt)
             kSlabTmaBufs * lpt * n) * 8;
 }
 constexpr int lpt_j(int T) { return T >= 256 ? 1 : 256 / T; }
+// k_pass_j (complex64, direct store): blocks of 128 threads for long lines, whose
+// last tiles then leave less of the chip idle.
+constexpr int lpt_jl(int T) { return T >= 32 ? (T >= 128 ? 1 : 128 / T) : lpt_j(T); }
 constexpr int lpt_rot(int T) { return T >= 64 ? 8 : (128 / T > 16 ? 128 / T : 16); }
 constexpr int lpt_c(int T, int want) { return T * want <= 1024 ? want : 0; }
 // Split-BF16 tensor-core variants exist for plans with a radix-16 stage and
