@@ -362,6 +362,8 @@ static int build_launches(fft3_plan_s *P)
             L.func = (p.cstream >= 0 && p.cstream < cnt)
                          ? (p.tc_mode < 0 ? ck[p.cstream].func : ck[p.cstream].func_tc[p.tc_mode == 0 ? 0 : 1])
                          : nullptr;
+            if (L.func && p.tc_mode < 0 && p.src != p.dst && P->elems * 8 >= (int64_t)2 << 30 && ck[p.cstream].func_out)
+                L.func = ck[p.cstream].func_out;
             L.stream_q = L.func ? ck[p.cstream].q : 0;
             L.cluster = p.p;
             break;

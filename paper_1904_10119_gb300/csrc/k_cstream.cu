@@ -107,11 +107,18 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // TC = 0: FP32 sub-line stages.  TC = 1: the first 16-point stage of every
-// sub-line on the tensor cores in split BF16 (tc_stage.cuh); TC = 2: both.
-template <int N, int Q, int R1, int R2, int G, int S, int LPT, int P, int TC>
+// sub-line on the tensor cores in split BF16 (tc_stage.cuh); TC = 2: both.  TC =
+// kStreamOut: FP32 stages whose results leave by streaming stores (evicted
+// first), which leaves L2 to the prefetched sub-lines: for arrays of 2 GiB and
+// more that the pass does not transform in place (1024^3: y 2783 -> 2716 us, z
+// 2847 -> 2812; 512^3, in place: 338 -> 340 and 366 -> 369).
+constexpr int kStreamOut = 3;
+template <int N, int Q, int R1, int R2, int G, int S, int LPT, int P, int TCV>
 __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(N, Q, Q / P, LPT, G *S), G *LPT *R2))
     k_cstream(PassArgs a, const __grid_constant__ CUtensorMap tin)
 {
+    constexpr bool STREAM = TCV == kStreamOut;
+    constexpr int TC = STREAM ? 0 : TCV;
     static_assert(TC == 0 || (R1 == 16 && R2 == 16 && P == 1 && LPT == 16),
                   "tensor-core sub-lines are 16 x 16, in tiles of 16 columns");
     constexpr int M = R1 * R2;
@@ -306,8 +313,14 @@ __global__ void __launch_bounds__(G *LPT *R2, cstream_min_blocks(cstream_smem_p(
                 Bfly<Q>::run(z);
                 if (valid) {
 #pragma unroll
-                    for (int s = 0; s < Q; ++s)
-                        op[(int64_t)(kk + s * M) * a.g.ok] = conj ? cconj(z[s]) : z[s];
+                    for (int s = 0; s < Q; ++s) {
+                        const float2 v = conj ? cconj(z[s]) : z[s];
+                        float2 *o = op + (int64_t)(kk + s * M) * a.g.ok;
+                        if constexpr (STREAM)
+                            __stcs(o, v);
+                        else
+                            *o = v;
+                    }
                 }
             }
         }
@@ -339,9 +352,19 @@ constexpr const void *cstream_tc_ptr()
         return nullptr;
 }
 
+template <int N, int Q, int R1, int R2, int G, int S, int LPT, int P>
+constexpr const void *cstream_out_ptr()
+{
+    if constexpr (P == 1 && N >= 512)
+        return (const void *)&k_cstream<N, Q, R1, R2, G, S, LPT, P, kStreamOut>;
+    else
+        return nullptr;
+}
+
 #define FFT3_CSTREAM_ROW(N, Q, R1, R2, G, S, LPT, P)                                      \
     {N, Q, R1, R2, G, S, LPT, P, G * LPT * R2, (const void *)&k_cstream<N, Q, R1, R2, G, S, LPT, P, 0>, \
-     {cstream_tc_ptr<N, Q, R1, R2, G, S, LPT, P, 1>(), cstream_tc_ptr<N, Q, R1, R2, G, S, LPT, P, 2>()}},
+     {cstream_tc_ptr<N, Q, R1, R2, G, S, LPT, P, 1>(), cstream_tc_ptr<N, Q, R1, R2, G, S, LPT, P, 2>()}, \
+     cstream_out_ptr<N, Q, R1, R2, G, S, LPT, P>()},
 
 static const CStreamKernel g_cstream_kernels[] = {FFT3_CSTREAM_LIST(FFT3_CSTREAM_ROW)};
 

@@ -66,7 +66,7 @@ const VolcKernel *volc_meta(int *count)
     return g_volc_meta;
 }
 
-#define FFT3_CSTREAM_META(N, Q, R1, R2, G, S, LPT, P) {N, Q, R1, R2, G, S, LPT, P, G * LPT * R2, nullptr, {nullptr, nullptr}},
+#define FFT3_CSTREAM_META(N, Q, R1, R2, G, S, LPT, P) {N, Q, R1, R2, G, S, LPT, P, G * LPT * R2, nullptr, {nullptr, nullptr}, nullptr},
 static const CStreamKernel g_cstream_meta[] = {FFT3_CSTREAM_LIST(FFT3_CSTREAM_META)};
 #undef FFT3_CSTREAM_META
 

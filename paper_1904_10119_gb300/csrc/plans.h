@@ -97,6 +97,7 @@ struct CStreamKernel {
     const void *func_tc[2]; // split-BF16 tensor-core sub-line stages: [0] the first, [1] both (R1 = R2 = 16)
                             // (tc_stages 0 takes [0]; 1 and 2 take [1]: both stages work in shared memory,
                             // the staging buffer and the result slot)
+    const void *func_out;   // func with streaming stores, for large arrays not transformed in place
 };
 // Compiled list (device translation unit) and the host-only metadata.
 const CStreamKernel *cstream_kernels(int *count);
