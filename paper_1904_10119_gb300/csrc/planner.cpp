@@ -1198,10 +1198,14 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
         // 30^3 x 10: 13.0 against 12.5; 96 x 96 x 1000: 211 against 87: the slab
         // kernel runs runtime radix lists).
         decomp = (int64_t)n0 * n1 <= 256 ? FFT3_SLAB_PENCIL : FFT3_PENCIL3;
-        // and with the blocked intermediate when it applies and the natural z lines
-        // would be at least 4 MiB apart (1024^3: 8.68 against 9.41 ms; at 512^3, 2 MiB
-        // apart, the natural layout measured 1.053 against 1.067 ms)
-        if (decomp == FFT3_PENCIL3 && s.opts.variant == FFT3_PPP_NATURAL && (int64_t)n0 * n1 * 8 >= (4ll << 20))
+        // and with the blocked intermediate when it applies, from 256 MiB on, unless the
+        // natural z lines are 512 points at 2 to 4 MiB (natural / blocked, us: 512 x 512 x
+        // 512 1026 / 1064, 256 x 1024 x 512 1047 / 1060; but 240 x 512 x 512 552 / 481,
+        // 480 x 512 x 512 1002 / 986, 512 x 512 x 1024 2136 / 2054, 1024 x 1024 x 512
+        // 4430 / 4133; below 256 MiB within 1%, or the natural order ahead by up to 5%)
+        const int64_t plane = (int64_t)n0 * n1 * 8;
+        if (decomp == FFT3_PENCIL3 && s.opts.variant == FFT3_PPP_NATURAL && plane * n2 >= (256ll << 20) &&
+            (plane >= (4ll << 20) || plane < (2ll << 20) || n2 >= 1024))
             s.opts.variant = FFT3_PPP_BLOCKED;
     }
     if (dtype == FFT3_C64_SPLITBF16_TC) {
