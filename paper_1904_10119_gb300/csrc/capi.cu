@@ -20,6 +20,7 @@ namespace fft3 {
 __global__ void k_pass_g(PassArgs a);
 __global__ void k_pass_g64(PassArgs a);
 __global__ void k_slab(PassArgs a);
+__global__ void k_slab_warp(PassArgs a);
 __global__ void k_vol(PassArgs a);
 __global__ void k_probe_pass(PassArgs a);
 __global__ void k_copy(const float2 *in, float2 *out, int64_t total);
@@ -326,7 +327,7 @@ static int build_launches(fft3_plan_s *P)
             break;
         }
         case PK_SLAB:
-            L.func = (const void *)&k_slab;
+            L.func = p.mixed ? (const void *)&k_slab_warp : (const void *)&k_slab;
             L.probe_g = natural_x(s);
             L.probe_n = s.n0;
             break;

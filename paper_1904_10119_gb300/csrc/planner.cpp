@@ -33,6 +33,7 @@
 #include "mixed_plans.h"
 #include "plans.h"
 #include "roots.cuh"
+#include "seg_plans.h"
 
 namespace fft3 {
 
@@ -816,6 +817,24 @@ static int make_vol_pass(Schedule *s, int d, int n, int p, const PassGeom &g, in
 // padded slab fit.
 static int slab_smem(int n0, int n1, int twlen) { return twlen * 8 + 2 * n1 * pitch_h(n0) * 8; }
 
+// The warp-register line plan of length n (N = R L over L / 2 lanes), if compiled.
+static bool warp_line(int n, LineChoice *lc)
+{
+#define FFT3_WARP_LINE(N, R, L)  \
+    if (n == N) {                \
+        *lc = LineChoice{};      \
+        lc->n = N;               \
+        lc->T = L / 2;           \
+        lc->nst = 2;             \
+        lc->rad[0] = R;          \
+        lc->rad[1] = L;          \
+        return true;             \
+    }
+    FFT3_SLABZ_WARP_PLANS(FFT3_WARP_LINE)
+#undef FFT3_WARP_LINE
+    return false;
+}
+
 static int make_slab_pass(Schedule *s, int n0, int n1, int64_t n2, int64_t batch, PassPlan *out,
                           std::string *err)
 {
@@ -824,6 +843,32 @@ static int make_slab_pass(Schedule *s, int n0, int n1, int64_t n2, int64_t batch
     q.dim = 3;
     q.src = BUF_IN;
     q.dst = BUF_OUT;
+    int64_t N = (int64_t)n0 * n1 * n2;
+    // one slab per tile; slabs indexed by (a = z, b = batch)
+    q.g = PassGeom{};
+    q.g.C = 1; q.g.A = n2; q.g.B = batch;
+    q.g.ij = 1; q.g.ic = 0; q.g.ia = (int64_t)n0 * n1; q.g.ib = N;
+    q.g.ok = 1; q.g.oc = 0; q.g.oa = q.g.ia; q.g.ob = N;
+    q.lpt = 1;
+    // Both sides of a compiled warp-register length: k_slab_warp (default radix order), but
+    // not for more small slabs than multiprocessors, which leave its 256 threads idle
+    // (16 x 16: 1024 slabs 12.4 us, with k_slab 10.3; 16 slabs 6.4, with k_slab 7.3).
+    const bool busy = (int64_t)n0 * n1 >= 384 || n2 * batch <= 152;
+    if (busy && s->opts.radix_order == 0 && warp_line(n0, &q.line) && warp_line(n1, &q.line2)) {
+        q.mixed = 1;
+        q.smem_bytes = n1 * (n0 | 1) * 8;
+        q.threads = 256;
+        for (int k = 0; k < 2; ++k) {
+            const int n = k ? n1 : n0;
+            std::vector<int64_t> m(n);
+            for (int i = 0; i < n; ++i)
+                m[i] = i;
+            q.tw_seg[k] = add_seg(s, n, std::move(m));
+        }
+        set_tiles(&q);
+        *out = q;
+        return FFT3_OK;
+    }
     int rc = choose_line(n0, s->opts.radix_order, false, &q.line, err);
     if (rc)
         return rc;
@@ -837,13 +882,6 @@ static int make_slab_pass(Schedule *s, int n0, int n1, int64_t n2, int64_t batch
     q.smem_bytes = slab_smem(n0, n1, twlen);
     if (q.smem_bytes > kSmemLimit)
         return FFT3_ERR_UNSUPPORTED_SIZE;
-    int64_t N = (int64_t)n0 * n1 * n2;
-    // one slab per tile; slabs indexed by (a = z, b = batch)
-    q.g = PassGeom{};
-    q.g.C = 1; q.g.A = n2; q.g.B = batch;
-    q.g.ij = 1; q.g.ic = 0; q.g.ia = (int64_t)n0 * n1; q.g.ib = N;
-    q.g.ok = 1; q.g.oc = 0; q.g.oa = q.g.ia; q.g.ob = N;
-    q.lpt = 1;
     int teams = std::max(1, std::max(n1, n0));
     int T = std::max(q.line.T, q.line2.T);
     // enough threads for one team of the longer line, up to 512 for the rest
@@ -1193,11 +1231,9 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
     }
     if (decomp == FFT3_AUTO) {
         // Fixed default when no cost model is loaded: pencil-pencil-pencil, whose
-        // passes are compiled for every length, but slab-pencil for slabs of at most
-        // 256 values, where one launch less counts (16^3: 10.0 against 12.2 us;
-        // 30^3 x 10: 13.0 against 12.5; 96 x 96 x 1000: 211 against 87: the slab
-        // kernel runs runtime radix lists).
-        decomp = (int64_t)n0 * n1 <= 256 ? FFT3_SLAB_PENCIL : FFT3_PENCIL3;
+        // passes are compiled for every length, but slab-pencil up to 1024 values,
+        // where a launch less counts (8^3: 5.7 against 7.0 us; 16^3: 8.2 against 7.3).
+        decomp = (int64_t)n0 * n1 * n2 * batch <= 1024 ? FFT3_SLAB_PENCIL : FFT3_PENCIL3;
         // and with the blocked intermediate when it applies, from 256 MiB on, unless the
         // natural z lines are 512 points at 2 to 4 MiB (natural / blocked, us: 512 x 512 x
         // 512 1026 / 1064, 256 x 1024 x 512 1047 / 1060; but 240 x 512 x 512 552 / 481,
@@ -1388,8 +1424,12 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
         int mode = s.opts.slab_mode;
         int twl = 2 * tw_slots_h(n0) + 2 * tw_slots_h(n1);
         bool fits_smem = slab_smem(n0, n1, twl) <= kSmemLimit;
-        if (mode == 0) // the L2-resident slab kernel measured slower than x and y passes (256^2 to 1024^2)
-            mode = fits_smem ? 1 : 3;
+        if (mode == 0)
+            // The L2-resident slab kernel measured slower than x and y passes (256^2 to
+            // 1024^2), and so does the shared-memory one, whose radix lists are data, once
+            // its values count for more than the launch it saves (slab / passes, us: 96 x 96
+            // x 1000 211 / 82, 54 x 18 x 576 x 4 66 / 25, 16 x 16 x 16 x 1000 57 / 37).
+            mode = fits_smem && N * batch <= (1 << 18) ? 1 : 3;
         PassPlan p;
         if (mode == 1 && fits_smem) {
             rc = make_slab_pass(&s, n0, n1, n2, batch, &p, err);

@@ -67,7 +67,7 @@ struct PassPlan {
     int64_t ntiles = 0, tiles_c = 0;
     int tc_mode = -1;           // split-BF16 tensor-core stages (tc_stages option); -1 = FP32 pass
     int volc = -1;              // PK_VOLC: index into the compiled volumetric list
-    int mixed = 0;              // PK_G: 1 / 2 = compiled mixed-radix pass, contiguous / strided lines (k_mixed.cuh)
+    int mixed = 0;              // PK_G, PK_G64: 1 / 2 = compiled mixed-radix pass, contiguous / strided lines; PK_SLAB: 1 = k_slab_warp
     int cstream = -1;           // PK_CSTREAM: index into the compiled streamed-pass list
     int chunk = 0;              // slabs per chunk of a two-stream pipelined slab stage (0 = one launch)
     bool pair_next = false;     // this pass and the next run chunk-interleaved on two streams
