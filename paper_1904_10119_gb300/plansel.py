@@ -26,12 +26,15 @@ SIZES = (16, 24, 32, 40, 48, 64, 80, 96, 128, 160, 192, 256, 320, 384, 512, 640,
 
 KINDS = ("line_contig", "line_contig_rotate", "line_strided", "line_runtime", "slab_smem", "slab_l2",
          "volumetric_split", "volumetric_split_fixed", "line_strided_stream", "line_strided_tma")
-N_FEATURES = 12 + len(KINDS) + 13
+N_FEATURES = 12 + len(KINDS) + 15
 # The fixed default is kept unless another plan is predicted faster by this much
-# (difference of log run times): most candidates of a shape run within a few per
-# cent of each other.  Mean regret on 30 small shapes over six runs: 0.021-0.027,
-# fixed default 0.032-0.036.
-MARGIN = 0.06
+# (difference of log run times) and by one standard deviation of the ensemble:
+# most candidates of a shape run within a few per cent of each other.  Mean regret
+# on 30 small shapes over ten runs: 0.031-0.048, fixed default 0.038-0.054 (with
+# targets to the shape's mean, not capped, and the mean prediction alone: 0.041-0.065).
+MARGIN = 0.02
+# Cap of the training targets, log of 1.35.
+CAP = 0.3
 
 
 def candidates():
@@ -92,6 +95,10 @@ def features(shape, batch, decomp, opts, schedule=None) -> np.ndarray:
     work = [math.log2(max(1, p["tiles"] * p["threads"])) for p in passes]
     f[k + 11] = float(np.mean(work))
     f[k + 12] = float(min(work))
+    # a slab kernel moves a whole slab in one block: its size and how many there are
+    if passes[0]["kind"].startswith("slab"):
+        f[k + 13] = math.log2(n0 * n1)
+        f[k + 14] = math.log2(n2 * batch)
     return f
 
 
@@ -128,25 +135,28 @@ def sample_shapes(count, seed, max_volume=1 << 24, exclude=()):
 
 
 def collect(shapes, batch=1, reps=3):
-    """Timing table: list of (shape, ms array over candidates)."""
+    """Timing table: list of (shape, ms array over candidates).  The first shape
+    is timed once before, for the clocks and the kernels' loading."""
+    if len(shapes):
+        time_shape(shapes[0], batch, reps)
     return [(s, time_shape(s, batch, reps)) for s in shapes]
 
 
 def to_xy(table, batch=1):
     """Features and targets: the log run time of each feasible candidate
-    relative to the mean log run time of the shape's candidates (only the
-    ranking within a shape matters for the choice)."""
+    relative to the fixed default's, at most CAP (what is far slower is never
+    chosen; how far needs none of the model's capacity)."""
     cands = candidates()
     X, y = [], []
     for shape, ms in table:
         valid = [(i, t) for i, t in enumerate(ms) if t > 0]
         if not valid:
             continue
-        mean_log = float(np.mean([math.log(t) for _, t in valid]))
+        base = ms[0] if ms[0] > 0 else min(t for _, t in valid)
         for i, t in valid:
             d, o = cands[i]
             X.append(features(shape, batch, d, o))
-            y.append(math.log(t) - mean_log)
+            y.append(min(math.log(t / base), CAP))
     return np.asarray(X, np.float32), np.asarray(y, np.float32)
 
 
@@ -178,9 +188,12 @@ class CostModel:
             self.mlps.append(net)
         return curve
 
-    def predict(self, X):
+    def members_predict(self, X):
         Z = (X - self.mu) / self.sd
-        return np.mean([net.predict(Z) for net in self.mlps], axis=0)
+        return np.stack([net.predict(Z) for net in self.mlps])
+
+    def predict(self, X):
+        return self.members_predict(X).mean(0)
 
     def close(self):
         for net in self.mlps:
@@ -189,8 +202,8 @@ class CostModel:
 
     def ranking(self, shape, batch=1):
         """Candidate indices the planner accepts for this shape, best
-        predicted first, the default ahead of them unless one is predicted
-        faster by more than MARGIN."""
+        first by the ensemble's mean difference from the default plus its
+        standard deviation, the default itself at -MARGIN."""
         cands = candidates()
         ok = []
         for i, (d, o) in enumerate(cands):
@@ -200,12 +213,13 @@ class CostModel:
             except fft3.Fft3Error:
                 pass
         X = np.stack([features(shape, batch, *cands[i]) for i in ok])
-        pred = self.predict(X)
-        order = [ok[j] for j in np.argsort(pred, kind="stable")]
-        if 0 in ok and pred.min() > pred[ok.index(0)] - MARGIN:
-            order.remove(0)
-            order.insert(0, 0)
-        return order
+        pred = self.members_predict(X)
+        if 0 not in ok:
+            return [ok[j] for j in np.argsort(pred.mean(0), kind="stable")]
+        gap = pred - pred[:, [ok.index(0)]]
+        score = gap.mean(0) + gap.std(0)
+        score[ok.index(0)] = -MARGIN
+        return [ok[j] for j in np.argsort(score, kind="stable")]
 
     def choose(self, shape, batch=1):
         return self.ranking(shape, batch)[0]
