@@ -48,12 +48,16 @@ enum fft3_dtype {
     FFT3_C64_SPLITBF16_TC = 1, /* radix-32 / radix-16 sub-DFTs as split-BF16 tensor-core GEMMs (hi + lo
                                   BF16 parts, three products), FP32 accumulation (options.tc_stages) */
     FFT3_C128_FP64 = 2         /* complex128 arrays (interleaved FP64 re, im; 16 bytes per element),
-                                  the paper's own precision (Section 4): each line is transformed in
-                                  64-bit block fixed point and rounded once to FP64 (error per pass
-                                  about 5e-17 of the line's norm), lines with infinities, NaN or
-                                  values outside 2^-895..2^1007 by FP64 butterflies.  Natural
-                                  pencil-pencil-pencil schedule (slab-pencil and FFT3_AUTO lower to it; volumetric, rotated,
-                                  blocked and permuted layouts are refused).  Buffers hold
+                                  the paper's own precision (Section 4).  A line is transformed in 64-bit
+                                  block fixed point and rounded once to FP64 where that is at least as
+                                  accurate as FP64 butterflies: largest real and largest imaginary part
+                                  within 2^5 of each other (or one all zeros; within 2^2 to 2^4 where the
+                                  line may be a single value), magnitudes in 2^-895..2^1007.  Other lines,
+                                  and those with infinities or NaN, run FP64 butterflies.  Error per pass,
+                                  of the line's norm: about 0.5e-16 for flat lines to 2.5e-16 for a spike
+                                  over a background at 4096 points; FP64 butterflies 1.5e-16 to 2.9e-16.
+                                  Natural pencil-pencil-pencil schedule (slab-pencil and FFT3_AUTO lower to
+                                  it; volumetric, rotated, blocked and permuted layouts are refused).  Buffers hold
                                   n0*n1*n2*batch complex128 values */
 };
 

@@ -12,17 +12,35 @@
 // 1/4, so the unit exponent rises by two per layer (see cmul62).  Radix 2, 3
 // and 8 = 4 * 2 layers fit the same rule; radix 5 takes one more halving.
 //
-// Error: a product is rounded to the unit, a halving truncates, so a layer adds
-// about one unit to a value, and passes half of the layers before it on (in
-// the rms, sqrt(4) / 4).  The result of a line of n points thus carries about
-// 1.3 units rms where its own rms is 2^59 / (crest * sqrt(n)) units and more,
-// crest = largest component / rms modulus of the line: 2^-55 at n = 1024 and
-// crest 2, against 2^-52 for the same stages in FP64.  Lines of 512 points and
-// more are shifted back up to full scale after the first stage (block floating
-// point), so a line that is one spike (crest sqrt(n)) is no exception.
-//
-// Lines with an infinity, a NaN or values so large or small that their exponent
-// cannot be carried (below 2^-895, above 2^1007) take the FP64 stages.
+// Error: products are rounded to the unit, shifts down truncate, so a layer adds
+// about one unit to a value.  After every stage but the last the line is shifted up
+// to full scale (block floating point), so scale that a line does not grow by is not
+// lost, and the result is rounded once to FP64.  Lists that lose more to their first
+// stage's scale (radix 10, 15, 32) round the shifts as well, and lists of run-time
+// length the conversion of the input too (256^3: 1.5% for the shifts, 10% for the
+// conversions).
+// Which lines take them: those in which no part is small enough to lose what
+// FP64 would keep.  Components share the largest one's exponent, so one that is
+// 2^-d of it keeps 59 - d bits.  Next to the largest values FP64 rounds to 53 bits
+// as well; what it keeps apart are real and imaginary parts, where no twiddle mixes
+// them.  So the largest real and the largest imaginary part must be within 2^5 of
+// each other, or one of them all zeros; and in a line that may be a single value
+// (a first-stage butterfly of zeros, or one stage in all), which FP64 carries
+// through the first element's additions as it is, so close that no stage shifts a
+// bit of it out (fix_exact_bits).  Lists that lose more of the scale, in a radix-32
+// first stage or over more than 2048 points from radix 5 on, are too coarse for
+// spikes over a background: there every first-stage butterfly must hold a value of
+// 2^-4 of the largest (fix_strict).
+// Measured on the host over every radix list of the plans (relative 2-norm per line
+// against long double; flat, real, tones, bumps, spectra, constants and spikes over
+// a background of 10^-1 to 10^-12): on the lines taken at most the error of the same
+// stages in FP64: flat lines 0.5e-16 against 2.9e-16, the hardest (4096 points, a
+// spike over 10^-12) 2.1e-16 against 2.4e-16.  With shifts up after the first stage
+// of some lists alone that spike had 5e-16 and more, and one over 1e-3 had 1.1e-15 at
+// 256 points as 8 x 8 x 4.
+// Other lines, and those with an infinity, a NaN or values so large or small
+// that their exponent cannot be carried (below 2^-895, above 2^1007), take the
+// FP64 stages.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -42,8 +60,19 @@ struct __align__(16) fix2 {
 FFT3_HD fix2 cadd(fix2 a, fix2 b) { return fix2{a.x + b.x, a.y + b.y}; }
 FFT3_HD fix2 csub(fix2 a, fix2 b) { return fix2{a.x - b.x, a.y - b.y}; }
 FFT3_HD fix2 mul_mi(fix2 a) { return fix2{a.y, -a.x}; }
-FFT3_HD fix2 quarter(fix2 a) { return fix2{a.x >> 2, a.y >> 2}; }
-FFT3_HD fix2 half(fix2 a) { return fix2{a.x >> 1, a.y >> 1}; }
+// Shifts down, rounded (RN) or not: rounding costs two instructions a component.
+template <bool RN>
+FFT3_HD fix2 quarter(fix2 a)
+{
+    constexpr int h = RN ? 2 : 0;
+    return fix2{(a.x + h) >> 2, (a.y + h) >> 2};
+}
+template <bool RN>
+FFT3_HD fix2 half(fix2 a)
+{
+    constexpr int h = RN ? 1 : 0;
+    return fix2{(a.x + h) >> 1, (a.y + h) >> 1};
+}
 FFT3_HD fix2 shl(fix2 a, int s)
 {
     return fix2{(long long)((unsigned long long)a.x << s), (long long)((unsigned long long)a.y << s)};
@@ -105,13 +134,13 @@ FFT3_HD constexpr long long fx_cos32(int m)
 }
 
 // a * w_32^M / 4, M known at compile time.
-template <int M>
+template <int M, bool RN>
 FFT3_HD fix2 mul_w32_4(fix2 a)
 {
     if constexpr (M == 0) {
-        return quarter(a);
+        return quarter<RN>(a);
     } else if constexpr (M == 8) {
-        return quarter(mul_mi(a));
+        return quarter<RN>(mul_mi(a));
     } else {
         constexpr long long c = fx_cos32(M), s = fx_cos32(M - 8); // w = c - i s
         return cmul62(a, root62{const_hi(c), const_lo(c), const_hi(-s), const_lo(-s)});
@@ -119,12 +148,13 @@ FFT3_HD fix2 mul_w32_4(fix2 a)
 }
 
 // In-register DFT_R of values with moduli below 2^60 (2^59 for R = 5); results
-// below 2^62.  scale(R): powers of two the result is scaled down by.
-template <int R>
+// below 2^62.  scale: powers of two the result is scaled down by; RN: shifts down
+// are rounded.
+template <int R, bool RN>
 struct BflyFix;
 
-template <>
-struct BflyFix<2> {
+template <bool RN>
+struct BflyFix<2, RN> {
     static constexpr int scale = 0;
     FFT3_HD static void run(fix2 *v)
     {
@@ -134,8 +164,8 @@ struct BflyFix<2> {
     }
 };
 
-template <>
-struct BflyFix<4> {
+template <bool RN>
+struct BflyFix<4, RN> {
     static constexpr int scale = 0;
     FFT3_HD static void run(fix2 *v)
     {
@@ -150,29 +180,29 @@ struct BflyFix<4> {
 
 // 8 = 2 * 4 and 16 = 4 * 4 by Eq. ct, as the floating-point butterflies, the
 // inner twiddles scaling by 1/4.
-template <>
-struct BflyFix<8> {
+template <bool RN>
+struct BflyFix<8, RN> {
     static constexpr int scale = 2;
     FFT3_HD static void run(fix2 *v)
     {
         fix2 e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
-        BflyFix<4>::run(e);
-        BflyFix<4>::run(o);
-        o[0] = mul_w32_4<0>(o[0]);
-        o[1] = mul_w32_4<4>(o[1]);
-        o[2] = mul_w32_4<8>(o[2]);
-        o[3] = mul_w32_4<12>(o[3]);
+        BflyFix<4, RN>::run(e);
+        BflyFix<4, RN>::run(o);
+        o[0] = mul_w32_4<0, RN>(o[0]);
+        o[1] = mul_w32_4<4, RN>(o[1]);
+        o[2] = mul_w32_4<8, RN>(o[2]);
+        o[3] = mul_w32_4<12, RN>(o[3]);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const fix2 q = quarter(e[k]);
+            const fix2 q = quarter<RN>(e[k]);
             v[k] = cadd(q, o[k]);
             v[k + 4] = csub(q, o[k]);
         }
     }
 };
 
-template <>
-struct BflyFix<16> {
+template <bool RN>
+struct BflyFix<16, RN> {
     static constexpr int scale = 2;
     FFT3_HD static void run(fix2 *v)
     {
@@ -182,27 +212,27 @@ struct BflyFix<16> {
 #pragma unroll
             for (int i1 = 0; i1 < 4; ++i1)
                 t[i0][i1] = v[i0 + 4 * i1];
-            BflyFix<4>::run(t[i0]);
+            BflyFix<4, RN>::run(t[i0]);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            t[0][k] = quarter(t[0][k]);
-        t[1][0] = quarter(t[1][0]);
-        t[1][1] = mul_w32_4<2>(t[1][1]);
-        t[1][2] = mul_w32_4<4>(t[1][2]);
-        t[1][3] = mul_w32_4<6>(t[1][3]);
-        t[2][0] = quarter(t[2][0]);
-        t[2][1] = mul_w32_4<4>(t[2][1]);
-        t[2][2] = mul_w32_4<8>(t[2][2]);
-        t[2][3] = mul_w32_4<12>(t[2][3]);
-        t[3][0] = quarter(t[3][0]);
-        t[3][1] = mul_w32_4<6>(t[3][1]);
-        t[3][2] = mul_w32_4<12>(t[3][2]);
-        t[3][3] = mul_w32_4<18>(t[3][3]);
+            t[0][k] = quarter<RN>(t[0][k]);
+        t[1][0] = quarter<RN>(t[1][0]);
+        t[1][1] = mul_w32_4<2, RN>(t[1][1]);
+        t[1][2] = mul_w32_4<4, RN>(t[1][2]);
+        t[1][3] = mul_w32_4<6, RN>(t[1][3]);
+        t[2][0] = quarter<RN>(t[2][0]);
+        t[2][1] = mul_w32_4<4, RN>(t[2][1]);
+        t[2][2] = mul_w32_4<8, RN>(t[2][2]);
+        t[2][3] = mul_w32_4<12, RN>(t[2][3]);
+        t[3][0] = quarter<RN>(t[3][0]);
+        t[3][1] = mul_w32_4<6, RN>(t[3][1]);
+        t[3][2] = mul_w32_4<12, RN>(t[3][2]);
+        t[3][3] = mul_w32_4<18, RN>(t[3][3]);
 #pragma unroll
         for (int k1 = 0; k1 < 4; ++k1) {
             fix2 c[4] = {t[0][k1], t[1][k1], t[2][k1], t[3][k1]};
-            BflyFix<4>::run(c);
+            BflyFix<4, RN>::run(c);
 #pragma unroll
             for (int k0 = 0; k0 < 4; ++k0)
                 v[k1 + 4 * k0] = c[k0];
@@ -211,18 +241,18 @@ struct BflyFix<16> {
 };
 
 // 32 = 2 * 16 (the radix-32 plan of 1024 points).
-template <int K>
+template <int K, bool RN>
 struct Tw32Fix {
     FFT3_HD static void run(fix2 *o)
     {
-        o[K] = mul_w32_4<K>(o[K]);
+        o[K] = mul_w32_4<K, RN>(o[K]);
         if constexpr (K + 1 < 16)
-            Tw32Fix<K + 1>::run(o);
+            Tw32Fix<K + 1, RN>::run(o);
     }
 };
 
-template <>
-struct BflyFix<32> {
+template <bool RN>
+struct BflyFix<32, RN> {
     static constexpr int scale = 4;
     FFT3_HD static void run(fix2 *v)
     {
@@ -232,12 +262,12 @@ struct BflyFix<32> {
             e[i] = v[2 * i];
             o[i] = v[2 * i + 1];
         }
-        BflyFix<16>::run(e);
-        BflyFix<16>::run(o);
-        Tw32Fix<0>::run(o);
+        BflyFix<16, RN>::run(e);
+        BflyFix<16, RN>::run(o);
+        Tw32Fix<0, RN>::run(o);
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-            const fix2 q = quarter(e[k]);
+            const fix2 q = quarter<RN>(e[k]);
             v[k] = cadd(q, o[k]);
             v[k + 16] = csub(q, o[k]);
         }
@@ -256,13 +286,13 @@ constexpr long long kFx1mS52 = 7604019954369499282ll; // 1 - sin(4 pi / 5)
 FFT3_HD long long fmulc(long long a, long long c) { return rmul62(a, const_hi(c), const_lo(c)); }
 
 // DFT_3 and DFT_5 in the forms of the floating-point butterflies.
-template <>
-struct BflyFix<3> {
+template <bool RN>
+struct BflyFix<3, RN> {
     static constexpr int scale = 0;
     FFT3_HD static void run(fix2 *v)
     {
         const fix2 s = cadd(v[1], v[2]), d = csub(v[1], v[2]);
-        const fix2 a = csub(v[0], half(s));
+        const fix2 a = csub(v[0], half<RN>(s));
         const fix2 b = fix2{d.x - fmulc(d.x, kFx1mS3), d.y - fmulc(d.y, kFx1mS3)};
         v[0] = cadd(v[0], s);
         v[1] = fix2{a.x + b.y, a.y - b.x};
@@ -270,8 +300,8 @@ struct BflyFix<3> {
     }
 };
 
-template <>
-struct BflyFix<5> {
+template <bool RN>
+struct BflyFix<5, RN> {
     static constexpr int scale = 1; // halves its inputs first
     // a1 = x0 + cos(2 pi/5) sa + cos(4 pi/5) sb, a2 the same with sa and sb swapped
     FFT3_HD static long long even(long long x0, long long sa, long long sb)
@@ -280,8 +310,8 @@ struct BflyFix<5> {
     }
     FFT3_HD static void run(fix2 *v)
     {
-        const fix2 x0 = half(v[0]);
-        const fix2 p1 = half(v[1]), p2 = half(v[2]), p3 = half(v[3]), p4 = half(v[4]);
+        const fix2 x0 = half<RN>(v[0]);
+        const fix2 p1 = half<RN>(v[1]), p2 = half<RN>(v[2]), p3 = half<RN>(v[3]), p4 = half<RN>(v[4]);
         const fix2 sa = cadd(p1, p4), da = csub(p1, p4), sb = cadd(p2, p3), db = csub(p2, p3);
         const fix2 a1 = fix2{even(x0.x, sa.x, sb.x), even(x0.y, sa.y, sb.y)};
         const fix2 a2 = fix2{even(x0.x, sb.x, sa.x), even(x0.y, sb.y, sa.y)};
@@ -342,7 +372,7 @@ FFT3_HD constexpr long long fx_sin_n(int m)
 
 // DFT_{A B} by Eq. ct (DFT_B, inner twiddles w_{AB}^{i0 k1} / 4, DFT_A); NT is
 // the table the twiddles come from (AB or a multiple).
-template <int A, int B, int NT, int I>
+template <int A, int B, int NT, int I, bool RN>
 struct CtFixTw {
     FFT3_HD static void run(fix2 (*t)[B])
     {
@@ -350,19 +380,19 @@ struct CtFixTw {
             constexpr int m = (I / B) * (I % B) * (NT / (A * B)) % NT;
             fix2 &v = t[I / B][I % B];
             if constexpr (m == 0) {
-                v = quarter(v);
+                v = quarter<RN>(v);
             } else {
                 constexpr long long c = fx_cos_n<NT>(m), s = fx_sin_n<NT>(m);
                 v = cmul62(v, root62{const_hi(c), const_lo(c), const_hi(-s), const_lo(-s)});
             }
-            CtFixTw<A, B, NT, I + 1>::run(t);
+            CtFixTw<A, B, NT, I + 1, RN>::run(t);
         }
     }
 };
 
-template <int A, int B, int NT>
+template <int A, int B, int NT, bool RN>
 struct BflyFixCt {
-    static constexpr int scale = BflyFix<B>::scale + 2 + BflyFix<A>::scale;
+    static constexpr int scale = BflyFix<B, RN>::scale + 2 + BflyFix<A, RN>::scale;
     FFT3_HD static void run(fix2 *v)
     {
         fix2 t[A][B];
@@ -371,36 +401,36 @@ struct BflyFixCt {
 #pragma unroll
             for (int i1 = 0; i1 < B; ++i1)
                 t[i0][i1] = v[i0 + A * i1];
-            BflyFix<B>::run(t[i0]);
+            BflyFix<B, RN>::run(t[i0]);
         }
-        CtFixTw<A, B, NT, 0>::run(t);
+        CtFixTw<A, B, NT, 0, RN>::run(t);
 #pragma unroll
         for (int k1 = 0; k1 < B; ++k1) {
             fix2 c[A];
 #pragma unroll
             for (int i0 = 0; i0 < A; ++i0)
                 c[i0] = t[i0][k1];
-            BflyFix<A>::run(c);
+            BflyFix<A, RN>::run(c);
 #pragma unroll
             for (int k0 = 0; k0 < A; ++k0)
                 v[k1 + B * k0] = c[k0];
         }
     }
 };
-template <>
-struct BflyFix<6> : BflyFixCt<2, 3, 12> {};
-template <>
-struct BflyFix<9> : BflyFixCt<3, 3, 9> {};
-template <>
-struct BflyFix<10> : BflyFixCt<2, 5, 10> {};
-template <>
-struct BflyFix<12> : BflyFixCt<4, 3, 12> {};
-template <>
-struct BflyFix<15> : BflyFixCt<3, 5, 15> {};
+template <bool RN>
+struct BflyFix<6, RN> : BflyFixCt<2, 3, 12, RN> {};
+template <bool RN>
+struct BflyFix<9, RN> : BflyFixCt<3, 3, 9, RN> {};
+template <bool RN>
+struct BflyFix<10, RN> : BflyFixCt<2, 5, 10, RN> {};
+template <bool RN>
+struct BflyFix<12, RN> : BflyFixCt<4, 3, 12, RN> {};
+template <bool RN>
+struct BflyFix<15, RN> : BflyFixCt<3, 5, 15, RN> {};
 
 // Normalisation between stages: `acc` is the OR of norm_word over the
 // components of a line; the line is shifted up by norm_shift(acc), which keeps
-// components below 2^61 (a line above that stays as it is).
+// components below 2^61 (a line within one bit of that stays as it is).
 FFT3_HD unsigned norm_word(long long v)
 {
     const int h = (int)(v >> 32);
@@ -417,7 +447,7 @@ FFT3_HD int clz32(unsigned v)
 FFT3_HD int norm_shift(unsigned acc)
 {
     const int l = clz32(acc) - 3;
-    return l > 0 ? l : 0;
+    return l > 1 ? l : 0;
 }
 
 // ------------------------------------------------------- conversions ---- //
@@ -434,15 +464,67 @@ FFT3_HD unsigned mag_word(double v)
     const unsigned h = (unsigned)(b >> 32) & 0x7fffffffu;
     return h ? h : ((unsigned)b != 0u ? 1u : 0u);
 }
-// Whether a line with this largest magnitude word takes the integer stages.
-FFT3_HD bool fix_ok(unsigned m) { return m == 0u || ((m >> 20) >= (unsigned)kFixMinExp && (m >> 20) <= (unsigned)kFixMaxExp); }
+// Largest magnitude words of the real and of the imaginary parts of some values.
+struct FixMag {
+    unsigned re, im;
+};
+FFT3_HD void mag_max(FixMag &m, double2 v)
+{
+    const unsigned a = mag_word(v.x), b = mag_word(v.y);
+    m.re = a > m.re ? a : m.re;
+    m.im = b > m.im ? b : m.im;
+}
+FFT3_HD unsigned mag_all(FixMag m) { return m.re > m.im ? m.re : m.im; }
+
+// What decides over a line, gathered over its first-stage butterflies.
+struct FixScan {
+    FixMag line{0u, 0u}; // the line's largest
+    unsigned least = ~0u; // the least of the butterflies' largest, those of zeros left out
+    bool zeros = false;  // whether there is a butterfly of zeros
+    FFT3_HD void add(FixMag m)
+    {
+        line.re = m.re > line.re ? m.re : line.re;
+        line.im = m.im > line.im ? m.im : line.im;
+        const unsigned all = mag_all(m);
+        zeros = zeros || all == 0u;
+        least = all != 0u && all < least ? all : least;
+    }
+};
+
+// How far (2^-bits) below the largest component another may lie without a stage of
+// radix scale `scale` shifting a bit of it out: a first stage has six bits to spare
+// and loses the butterfly's scale, a later one has eight (from the shift up) and
+// loses two more.
+FFT3_HD constexpr int fix_exact_bits(int scale) { return 6 - scale; }
+
+// Whether a list whose first stage has this scale rounds its shifts down.
+FFT3_HD constexpr bool fix_rounds(int scale) { return scale > 2; }
+
+// Whether a list of n points that starts with radix R takes only lines with a large
+// value in every first-stage butterfly.
+FFT3_HD constexpr bool fix_strict(int n, int R) { return R == 32 || (R == 5 && n > 2048); }
+
+// Whether a line takes the integer stages; exact: the least fix_exact_bits of its
+// stages.  Holds for a line when it holds for every part of its butterflies (least,
+// zeros) with the whole line's `line`.
+FFT3_HD bool fix_ok(const FixScan &s, bool strict, int exact)
+{
+    const unsigned m = mag_all(s.line), e = m >> 20;
+    if (m == 0u)
+        return true;
+    if (e < (unsigned)kFixMinExp || e > (unsigned)kFixMaxExp || (strict && s.least < m - (4u << 20)))
+        return false;
+    const unsigned low = m - ((s.zeros && exact < 5 ? (unsigned)exact : 5u) << 20);
+    return (s.line.re == 0u || s.line.re >= low) && (s.line.im == 0u || s.line.im >= low);
+}
 
 // Exponent field the line's values are scaled by (any of the range for a zero
 // line: a zero's mantissa is then shifted out).
 FFT3_HD int fix_emax(unsigned m) { return m ? (int)(m >> 20) : 1023; }
 
-// v in units of 2^(emax - 1023 - 58): components below 2^59, moduli below 2^60
+// v in units of 2^(emax - 1023 - 58), rounded (RN) or truncated: components below 2^59, moduli below 2^60
 // (emax: exponent field of the line's largest component).
+template <bool RN>
 FFT3_HD long long to_fix(double v, int emax)
 {
     unsigned long long b;
@@ -451,7 +533,10 @@ FFT3_HD long long to_fix(double v, int emax)
     const int e = (int)((hi >> 20) & 0x7ffu);
     unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b;
     const int d = emax - e;
-    m = (m << 6) >> (d < 63 ? d : 63);
+    m <<= 6;
+    if (RN)
+        m += (1ull << (d < 62 ? d : 62)) >> 1;
+    m >>= d < 63 ? d : 63;
     return (int)hi < 0 ? -(long long)m : (long long)m;
 }
 

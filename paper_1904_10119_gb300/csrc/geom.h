@@ -41,6 +41,8 @@ enum : unsigned {
 
 constexpr int kMaxStages = 12;
 
+constexpr int kFix64LineWords = 7; // shared words k_pass_g64 keeps per line (FixLineState)
+
 // A line transform with its radix list known only at run time.
 struct LineRt {
     int n, T, nst, tw_off; // tw_off: offset of its stage-major table inside the pass table

@@ -74,13 +74,14 @@ __global__ void k_pass_g(PassArgs a)
 // ---------------------------------------------------------- k_pass_g64 -- //
 // The complex128 path: the same tile in 64-bit block fixed point (fix64.cuh),
 // every line normalised after each of its stages.  Per line the block keeps
-// its largest magnitude word, the sum of its shifts and three rotating words
-// for the normalisation (stage s fills slot s % 3, reads the one before and
-// clears the one after).  A tile with a line the integers do not take runs the
-// FP64 stages on the same buffers, its twiddles read from global memory.
+// its largest magnitude words, the least of its first-stage butterflies', the sum of
+// its shifts and three rotating words for the normalisation (stage s fills slot s % 3, reads the one before and clears
+// the one after).  A tile with a line the integers do not take runs the FP64
+// stages on the same buffers, its twiddles read from global memory.
 struct FixLineState {
-    unsigned *mx;  // [lpt]
-    int *up;       // [lpt]
+    FixMag *line;  // [lpt]
+    unsigned *least; // [lpt], complemented
+    int *up;       // [lpt]; during the scan: whether a first-stage butterfly is all zeros
     unsigned *nrm; // [3][lpt]
 };
 
@@ -97,18 +98,18 @@ __device__ __forceinline__ void stage_fix_rt(const LineRt &L, int NS, int t, con
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const double2 x = reinterpret_cast<const double2 *>(src)[padpos(q + r * NB)];
-                v[r] = fix2{to_fix(x.x, emax), to_fix(x.y, emax)};
+                v[r] = fix2{to_fix<true>(x.x, emax), to_fix<true>(x.y, emax)};
             }
         } else {
 #pragma unroll
             for (int r = 0; r < R; ++r)
                 v[r] = shl(src[padpos(q + r * NB)], up);
-            v[0] = quarter(v[0]);
+            v[0] = quarter<true>(v[0]);
 #pragma unroll
             for (int r = 1; r < R; ++r)
                 v[r] = cmul62(v[r], tw[(r - 1) * NS + k]);
         }
-        BflyFix<R>::run(v);
+        BflyFix<R, true>::run(v);
         const int base = (q / NS) * NS * R + k;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -136,7 +137,7 @@ __device__ __forceinline__ fix2 *run_stages_fix(const LineRt &L, int lpt, int P,
             for (int l = team; l < lpt; l += nteams) {
                 const fix2 *src = cur + l * P;
                 fix2 *dst = nxt + l * P;
-                const int emax = fix_emax(st.mx[l]);
+                const int emax = fix_emax(mag_all(st.line[l]));
                 const int up = s ? norm_shift(prev[l]) : 0;
                 if (t == 0) {
                     clear[l] = 0;
@@ -179,35 +180,45 @@ __global__ void __launch_bounds__(512) k_pass_g64(PassArgs a) // kMaxThreadsG64
     root62 *tw = reinterpret_cast<root62 *>(g_smem_raw);
     fix2 *b0 = reinterpret_cast<fix2 *>(tw + tw_slots(a.tw_len)), *b1 = b0 + lpt * P;
     unsigned *words = reinterpret_cast<unsigned *>(b1 + lpt * P);
-    const FixLineState st{words, reinterpret_cast<int *>(words + lpt), words + 2 * lpt};
+    const FixLineState st{reinterpret_cast<FixMag *>(words), words + 2 * lpt, reinterpret_cast<int *>(words + 3 * lpt),
+                          words + 4 * lpt};
     const root62 *twg = reinterpret_cast<const root62 *>(a.tw_fix);
     for (int i = threadIdx.x; i < a.tw_len; i += blockDim.x)
         tw[i] = twg[i];
     pdl_wait();
-    int scale = 0; // powers of two the stages scale down by
-    for (int s = 0; s < L.nst; ++s)
+    int scale = 0, exact = fix_exact_bits(0); // powers of two the stages scale down by; least fix_exact_bits
+    for (int s = 0; s < L.nst; ++s) {
         scale += fix_scale_rt(L.rad[s]) + (s ? 2 : 0);
+        exact = min(exact, fix_exact_bits(fix_scale_rt(L.rad[s])));
+    }
     const int nteams = blockDim.x / L.T, team = threadIdx.x / L.T, t = threadIdx.x - team * L.T;
+    const int R0 = L.nst ? L.rad[0] : 1, NB0 = n / R0; // first-stage butterflies
     for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
         __syncthreads();
         const TileG tg = tile_g(a, tile);
-        for (int i = threadIdx.x; i < 5 * lpt; i += blockDim.x)
+        for (int i = threadIdx.x; i < kFix64LineWords * lpt; i += blockDim.x)
             words[i] = 0;
         tile_g_load(a, tg, reinterpret_cast<const double2 *>(a.in), reinterpret_cast<double2 *>(b0), n, P);
         __syncthreads();
         if (team < nteams)
             for (int l = team; l < lpt; l += nteams) {
-                unsigned m = 0;
-                for (int j = t; j < n; j += L.T) {
-                    const double2 v = reinterpret_cast<const double2 *>(b0)[l * P + padpos(j)];
-                    m = max(m, max(mag_word(v.x), mag_word(v.y)));
+                FixScan scan;
+                for (int q = t; q < NB0; q += L.T) {
+                    FixMag m{0u, 0u};
+                    for (int r = 0; r < R0; ++r)
+                        mag_max(m, reinterpret_cast<const double2 *>(b0)[l * P + padpos(q + r * NB0)]);
+                    scan.add(m);
                 }
-                atomicMax(st.mx + l, m);
+                atomicMax(&st.line[l].re, scan.line.re);
+                atomicMax(&st.line[l].im, scan.line.im);
+                atomicMax(st.least + l, ~scan.least);
+                if (scan.zeros || L.nst == 1)
+                    st.up[l] = 1;
             }
         __syncthreads();
         bool bad = false;
         for (int l = threadIdx.x; l < lpt; l += blockDim.x)
-            bad = bad || !fix_ok(st.mx[l]);
+            bad = bad || !fix_ok(FixScan{st.line[l], ~st.least[l], st.up[l] != 0}, fix_strict(n, R0), exact);
         if (__syncthreads_or(bad)) {
             tile_g64_fp64(a, tg, reinterpret_cast<double2 *>(b0), reinterpret_cast<double2 *>(b1), P);
             continue;
@@ -218,7 +229,7 @@ __global__ void __launch_bounds__(512) k_pass_g64(PassArgs a) // kMaxThreadsG64
             const fix2 v = res[slot];
             if (none)
                 return reinterpret_cast<const double2 *>(res)[slot];
-            const int sh = fix_emax(st.mx[l]) - 1081 + scale - st.up[l];
+            const int sh = fix_emax(mag_all(st.line[l])) - 1081 + scale - st.up[l];
             return make_double2(from_fix(v.x, sh), from_fix(v.y, sh));
         });
     }

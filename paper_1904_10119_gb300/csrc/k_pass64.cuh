@@ -9,16 +9,18 @@
 //   k_pass_c64  strided lines (ic == 1, oc == 1), tiles of 8 adjacent
 //               columns (128-byte rows), position-major shared layout.
 // A tile: every thread loads the inputs of its first butterflies, the line's
-// largest exponent is reduced in shared memory, the inputs become integers, and
-// the stages run as in FP32, the last one rounding to FP64.  A tile with a line
+// largest magnitudes are reduced in shared memory, the inputs become integers, and
+// the stages run as in FP32, the line shifted up to full scale after each, the last
+// one rounding to FP64.  A tile with a line
 // that the integers do not take (fix_ok) is redone from its input by the FP64
 // stages; every thread learns that at the barrier that ends the first stage,
 // before anything has been stored.
 //
 // What bounds it: latency at 16 warps per SM (128 registers: 16 values of four
 // words each) and the integer pipe, 48% busy; the FP64 pipe carries only half of
-// the final roundings.  256^3: 572 us, 2.8 TB/s per pass, against 2502 us with
-// FP64 stages (2 lanes per clock and SM).  Tried: radix-8 plans (24 warps, one
+// the final roundings.  256^3: 580 us, 2.8 TB/s per pass, against 2502 us with
+// FP64 stages (2 lanes per clock and SM); without the shifts up, which dominated
+// lines need, 567.  Tried: radix-8 plans (24 warps, one
 // exchange more) 671 us; up to 168 registers (12 warps) 630 us.
 // The runtime-radix kernel (k_pass_g64) covers the other lengths.
 #pragma once
@@ -85,31 +87,51 @@ __device__ __forceinline__ unsigned char *smem64()
     return s64_raw;
 }
 
-// Powers of two the integer stages of a radix list scale down by.
+// Powers of two the integer stages of a radix list scale down by, and the least of their fix_exact_bits.
 template <class Rad>
 struct FixScale;
 template <int R>
 struct FixScale<Radices<R>> {
-    static constexpr int value = BflyFix<R>::scale;
+    static constexpr int value = BflyFix<R, false>::scale;
+    static constexpr int exact = fix_exact_bits(BflyFix<R, false>::scale);
 };
 template <int R, int R2, int... Rest>
 struct FixScale<Radices<R, R2, Rest...>> {
-    static constexpr int value = BflyFix<R>::scale + 2 + FixScale<Radices<R2, Rest...>>::value;
+    using Later = FixScale<Radices<R2, Rest...>>;
+    static constexpr int value = BflyFix<R, false>::scale + 2 + Later::value;
+    static constexpr int exact = fix_exact_bits(BflyFix<R, false>::scale) < Later::exact ? fix_exact_bits(BflyFix<R, false>::scale)
+                                                                                  : Later::exact;
 };
 
+// OR of a line's normalisation words over the adjacent lanes that hold it, into
+// the line's shared slot.
+template <int SEG>
+__device__ __forceinline__ void norm_out(unsigned acc, unsigned *slot)
+{
+#pragma unroll
+    for (int o = 1; o < SEG; o <<= 1)
+        acc |= __shfl_xor_sync(0xffffffffu, acc, o);
+    if (SEG == 1 || (threadIdx.x & (SEG - 1)) == 0)
+        atomicOr(slot, acc);
+}
+
 // Stages after the first: shared buffer to shared buffer, the last to `dst`.
-// `up` shifts the first of them's inputs (normalisation).
-template <int N, int T, int NS, class Rad>
+// `nrm` is the slot the stage before left its normalisation word in, the next
+// stage's is NSTEP words on.
+template <int N, int T, int NS, class Rad, int SEG, int NSTEP, bool RN>
 struct FixRest;
-template <int N, int T, int NS, int R, int... Rest>
-struct FixRest<N, T, NS, Radices<R, Rest...>> {
+template <int N, int T, int NS, int R, int... Rest, int SEG, int NSTEP, bool RN>
+struct FixRest<N, T, NS, Radices<R, Rest...>, SEG, NSTEP, RN> {
     static constexpr bool LAST = sizeof...(Rest) == 0;
-    template <bool UP, class Sm, class Dst>
-    __device__ __forceinline__ static void run(int t, const Sm &sm, const Dst &dst, const root62 *tw, int up)
+    template <class Sm>
+    __device__ __forceinline__ static void run(int t, const Sm &sm, FixStore dst, const root62 *tw, unsigned *nrm)
     {
         constexpr int NB = N / R, BPT = (NB + T - 1) / T;
         constexpr bool FULL = NB % T == 0;
+        const int up = norm_shift(*nrm);
+        dst.sh -= up;
         fix2 v[BPT][R];
+        unsigned acc = 0;
 #pragma unroll
         for (int b = 0; b < BPT; ++b) {
             const int q = t + b * T;
@@ -126,29 +148,32 @@ struct FixRest<N, T, NS, Radices<R, Rest...>> {
             const int q = t + b * T;
             if (FULL || q < NB) {
                 const int k = q % NS;
-                if constexpr (UP) {
+                if (up > 0) {
 #pragma unroll
                     for (int r = 0; r < R; ++r)
                         v[b][r] = shl(v[b][r], up);
                 }
-                v[b][0] = quarter(v[b][0]);
+                v[b][0] = quarter<RN>(v[b][0]);
 #pragma unroll
                 for (int r = 1; r < R; ++r)
                     v[b][r] = cmul62(v[b][r], tw[(r - 1) * NS + k]);
-                BflyFix<R>::run(v[b]);
+                BflyFix<R, RN>::run(v[b]);
                 const int base = (q / NS) * NS * R + k;
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    if constexpr (LAST)
+                    if constexpr (LAST) {
                         dst(base + r * NS, v[b][r]);
-                    else
+                    } else {
                         sm(base + r * NS, v[b][r]);
+                        acc |= norm_word(v[b][r].x) | norm_word(v[b][r].y);
+                    }
                 }
             }
         }
         if constexpr (!LAST) {
+            norm_out<SEG>(acc, nrm + NSTEP);
             __syncthreads();
-            FixRest<N, T, NS * R, Radices<Rest...>>::template run<false>(t, sm, dst, tw + (R - 1) * NS, 0);
+            FixRest<N, T, NS * R, Radices<Rest...>, SEG, NSTEP, RN>::run(t, sm, dst, tw + (R - 1) * NS, nrm + NSTEP);
         }
     }
 };
@@ -161,33 +186,28 @@ __device__ __noinline__ void tile_fp64(int t, G64Load src, Sm sm, G64Store dst, 
     EngineFixed<N, T, 1, Rad>::template run<true, false>(t, src, sm, dst, tw);
 }
 
-// Lines that are normalised after their first stage (UP): where three stages or
-// more follow each other or odd radices waste part of the scale.
-template <int N, class Rad>
-struct FixNormalise;
-template <int N, int... Rs>
-struct FixNormalise<N, Radices<Rs...>> {
-    static constexpr bool value = sizeof...(Rs) > 1 && (N >= 512 || (N & (N - 1)) != 0);
-};
-
-// One tile's line of this thread: `mx` and `nrm` are this line's shared slots
-// (zero on entry), SEG > 1 the adjacent lanes of a warp that hold one line.
-template <int N, int T, class Rad, int SEG>
+// One tile's line of this thread: `slot` is the line's first shared word (largest
+// magnitude words of the real and the imaginary parts, then a normalisation word
+// per stage but the last; zero on entry), the following ones NSTEP words apart;
+// SEG > 1 the adjacent lanes of a warp that hold one line.
+template <int N, int T, class Rad, int SEG, int NSTEP>
 struct FixTile;
-template <int N, int T, int R, int... Rest, int SEG>
-struct FixTile<N, T, Radices<R, Rest...>, SEG> {
+template <int N, int T, int R, int... Rest, int SEG, int NSTEP>
+struct FixTile<N, T, Radices<R, Rest...>, SEG, NSTEP> {
     using Rad = Radices<R, Rest...>;
     template <class SmF, class SmD>
     __device__ __forceinline__ static void run(int t, const G64Load &src, const SmF &sm, const SmD &smd,
                                                const G64Store &dst, const root62 *tw, const double2 *twd,
-                                               unsigned *mx, unsigned *nrm)
+                                               unsigned *slot)
     {
         constexpr int NB = N / R, BPT = (NB + T - 1) / T;
         constexpr bool FULL = NB % T == 0, ONE = sizeof...(Rest) == 0;
+        constexpr bool RN = fix_rounds(BflyFix<R, false>::scale);
         static_assert(!ONE || T == 1, "a line of one stage belongs to one thread");
-        constexpr bool UP = FixNormalise<N, Rad>::value;
         double2 x[BPT][R];
-        unsigned m = 0;
+        FixScan scan;
+        scan.zeros = ONE;
+        FixMag &line = scan.line;
 #pragma unroll
         for (int b = 0; b < BPT; ++b) {
             const int q = t + b * T;
@@ -195,23 +215,31 @@ struct FixTile<N, T, Radices<R, Rest...>, SEG> {
 #pragma unroll
                 for (int r = 0; r < R; ++r)
                     x[b][r] = src(q + r * NB);
+                FixMag m{0u, 0u};
 #pragma unroll
                 for (int r = 0; r < R; ++r)
-                    m = max(m, max(mag_word(x[b][r].x), mag_word(x[b][r].y)));
+                    mag_max(m, x[b][r]);
+                scan.add(m);
             }
         }
         if constexpr (!ONE) {
 #pragma unroll
-            for (int o = 1; o < SEG; o <<= 1)
-                m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (SEG == 1 || (threadIdx.x & (SEG - 1)) == 0)
-                atomicMax(mx, m);
+            for (int o = 1; o < SEG; o <<= 1) {
+                line.re = max(line.re, __shfl_xor_sync(0xffffffffu, line.re, o));
+                line.im = max(line.im, __shfl_xor_sync(0xffffffffu, line.im, o));
+            }
+            if (SEG == 1 || (threadIdx.x & (SEG - 1)) == 0) {
+                atomicMax(slot, line.re);
+                atomicMax(slot + NSTEP, line.im);
+            }
             __syncthreads();
-            m = *mx;
+            line.re = slot[0];
+            line.im = slot[NSTEP];
         }
-        const bool ok = fix_ok(m);
-        const int emax = fix_emax(m);
-        if (ONE && !ok) {
+        const bool ok = fix_ok(scan, fix_strict(N, R), FixScale<Rad>::exact);
+        const int emax = fix_emax(mag_all(line));
+        // 2 and 4 points are additions alone, exact in FP64 more often than not
+        if (ONE && (R == 2 || R == 4 || !ok)) {
             Bfly<R>::run(x[0]);
 #pragma unroll
             for (int r = 0; r < R; ++r)
@@ -219,7 +247,7 @@ struct FixTile<N, T, Radices<R, Rest...>, SEG> {
             return;
         }
         unsigned acc = 0;
-        FixStore out{dst, emax - 1081 + FixScale<Rad>::value};
+        const FixStore out{dst, emax - 1081 + FixScale<Rad>::value};
 #pragma unroll
         for (int b = 0; b < BPT; ++b) {
             const int q = t + b * T;
@@ -227,34 +255,26 @@ struct FixTile<N, T, Radices<R, Rest...>, SEG> {
                 fix2 v[R];
 #pragma unroll
                 for (int r = 0; r < R; ++r)
-                    v[r] = fix2{to_fix(x[b][r].x, emax), to_fix(x[b][r].y, emax)};
-                BflyFix<R>::run(v);
+                    v[r] = fix2{to_fix<false>(x[b][r].x, emax), to_fix<false>(x[b][r].y, emax)};
+                BflyFix<R, RN>::run(v);
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    if constexpr (ONE)
+                    if constexpr (ONE) {
                         out(r, v[r]);
-                    else
+                    } else {
                         sm(q * R + r, v[r]);
-                    if constexpr (UP)
                         acc |= norm_word(v[r].x) | norm_word(v[r].y);
+                    }
                 }
             }
         }
         if constexpr (!ONE) {
-            if constexpr (UP) {
-#pragma unroll
-                for (int o = 1; o < SEG; o <<= 1)
-                    acc |= __shfl_xor_sync(0xffffffffu, acc, o);
-                if (SEG == 1 || (threadIdx.x & (SEG - 1)) == 0)
-                    atomicOr(nrm, acc);
-            }
+            norm_out<SEG>(acc, slot + 2 * NSTEP);
             if (__syncthreads_or(!ok)) {
                 tile_fp64<N, T, Rad>(t, src, smd, dst, twd);
                 return;
             }
-            const int up = UP ? norm_shift(*nrm) : 0;
-            out.sh -= up;
-            FixRest<N, T, R, Radices<Rest...>>::template run<UP>(t, sm, out, tw + (R - 1), up);
+            FixRest<N, T, R, Radices<Rest...>, SEG, NSTEP, RN>::run(t, sm, out, tw + (R - 1), slot + 2 * NSTEP);
         }
     }
 };
@@ -265,7 +285,8 @@ template <int N, int T, class Rad, int LPT, int G, bool LINES, int SH = 4, int P
 __device__ __forceinline__ void pass64(const PassArgs &a)
 {
     constexpr int GT = T * LPT, NT = GT * G;
-    __shared__ unsigned slots[2][2][G * LPT]; // [tile parity][largest magnitude word, normalisation word][line]
+    constexpr int WORDS = 1 + Rad::count; // FixTile's words of a line
+    __shared__ unsigned slots[2][WORDS][G * LPT]; // [tile parity][word][line]
     root62 *tw = reinterpret_cast<root62 *>(smem64());
     unsigned char *buf = smem64() + (size_t)tw_slots(a.tw_len) * 16;
     const root62 *twg = reinterpret_cast<const root62 *>(a.tw_fix);
@@ -283,7 +304,7 @@ __device__ __forceinline__ void pass64(const PassArgs &a)
     const bool conj = a.conj != 0;
     int par = 0;
     for (int64_t tile0 = (int64_t)blockIdx.x * G; tile0 < a.ntiles; tile0 += (int64_t)gridDim.x * G, par ^= 1) {
-        for (int i = threadIdx.x; i < 2 * G * LPT; i += NT)
+        for (int i = threadIdx.x; i < WORDS * G * LPT; i += NT)
             slots[par][i / (G * LPT)][i % (G * LPT)] = 0;
         __syncthreads();
         const bool live = G == 1 || tile0 + g < a.ntiles;
@@ -292,15 +313,15 @@ __device__ __forceinline__ void pass64(const PassArgs &a)
         const bool valid = live && c < a.g.C;
         const G64Load src{in + c * a.g.ic + id.a * a.g.ia + id.b * a.g.ib, LINES ? 1 : a.g.ij, valid, conj};
         const G64Store dst{out + c * a.g.oc + id.a * a.g.oa + id.b * a.g.ob, LINES ? 1 : a.g.ok, valid, conj};
-        unsigned *mx = &slots[par][0][g * LPT + l], *nrm = &slots[par][1][g * LPT + l];
+        unsigned *slot = &slots[par][0][g * LPT + l];
         if constexpr (LINES) {
             const Smem64Line<fix2, SH> sm{reinterpret_cast<fix2 *>(buf) + l * PITCH};
             const Smem64Line<double2, SH> smd{reinterpret_cast<double2 *>(buf) + l * PITCH};
-            FixTile<N, T, Rad, SEG>::run(t, src, sm, smd, dst, tw, twd, mx, nrm);
+            FixTile<N, T, Rad, SEG, G * LPT>::run(t, src, sm, smd, dst, tw, twd, slot);
         } else {
             const Smem64Col<fix2, LPT> sm{reinterpret_cast<fix2 *>(buf) + g * (LPT * N) + l};
             const Smem64Col<double2, LPT> smd{reinterpret_cast<double2 *>(buf) + g * (LPT * N) + l};
-            FixTile<N, T, Rad, SEG>::run(t, src, sm, smd, dst, tw, twd, mx, nrm);
+            FixTile<N, T, Rad, SEG, G * LPT>::run(t, src, sm, smd, dst, tw, twd, slot);
         }
     }
 }

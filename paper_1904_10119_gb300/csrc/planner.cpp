@@ -252,8 +252,8 @@ void generic_launch_shape_elem(int n, int T, bool strided, int tw_len, int esize
     int l = strided ? 128 / esize : std::max(1, 256 / T);
     while (l > 1 && T * l > (esize == 16 ? kMaxThreadsG64 : 1024))
         l /= 2;
-    // complex128: five words per line for the block fixed point (k_pass_g64)
-    const int state = esize == 16 ? 5 * 4 : 0;
+    // complex128: a line's words for the block fixed point (k_pass_g64)
+    const int state = esize == 16 ? kFix64LineWords * 4 : 0;
     auto bytes = [&](int ll) { return tw_slots_h(tw_len) * esize + ll * (2 * P * esize + state); };
     while (l > 1 && bytes(l) > kSmemLimit)
         l /= 2;

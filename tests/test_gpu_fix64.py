@@ -11,7 +11,7 @@ from paper_1904_10119_gb300 import fft3, synth
 pytestmark = pytest.mark.gpu
 
 
-def _passes(z):
+def _passes(z, **opts):
     """The rows of z as contiguous lines (pass 0 of n x lines) and as strided
     columns (pass 1 of lines x n, in place on the output), one pass alone."""
     lines, n = z.shape
@@ -19,7 +19,7 @@ def _passes(z):
     for dims, k, a in (((n, lines, 1), 0, z), ((lines, n, 1), 1, z.T)):
         x = torch.from_numpy(np.ascontiguousarray(a)).cuda()
         out = torch.full_like(x, complex(float("nan"), float("nan"))) if k == 0 else x.clone()
-        plan = fft3.Plan(*dims, dtype=fft3.FFT3_C128_FP64)
+        plan = fft3.Plan(*dims, dtype=fft3.FFT3_C128_FP64, **opts)
         fft3.fft3_plan_execute_pass(plan.handle, k, x.data_ptr(), out.data_ptr())
         torch.cuda.synchronize()
         assert plan.check() == 0, fft3.last_error()
@@ -96,3 +96,43 @@ def test_lines_left_to_fp64(n):
             # 1e-310 is held to 2^-1074 only: 4e-324 * sqrt(n) of absolute error
             assert np.linalg.norm((a - b) * 2.0 ** -60) <= 1e-15 * np.linalg.norm(b * 2.0 ** -60) or \
                 np.abs(a - b).max() <= 5e-324 * 4 * n
+
+
+@pytest.mark.parametrize("order", range(4))
+@pytest.mark.parametrize("n", [48, 64, 120, 128, 256, 375, 512, 600, 1024, 2048])
+def test_dominated_lines_keep_fp64_accuracy(n, order):
+    """One value just above a power of two over a small background, and its
+    transform (a constant with noise), under every radix order: no further off
+    than FP64 stages, at most 33 roundings of 2^-53 / sqrt(3) (log2 n levels of two
+    additions, three products per twiddle), each of the value's size at most."""
+    rng = np.random.default_rng(n)
+    noise = rng.uniform(-1, 1, (9, n)) + 1j * rng.uniform(-1, 1, (9, n))
+    for bg in (0.1, 1e-3, 1e-12):
+        for dc in (False, True):
+            z = bg * noise
+            if dc:
+                z += 1.01 + 0.7j
+            else:
+                z[np.arange(9), rng.integers(0, n, 9)] = 1.01 + 0.3j
+            ref = np.fft.fft(z.astype(np.clongdouble), axis=1)
+            for got in _passes(z, radix_order=order):
+                err = np.sqrt((np.abs(got.astype(np.clongdouble) - ref) ** 2).sum(axis=1) / (np.abs(ref) ** 2).sum(axis=1))
+                assert err.max() <= 3.7e-16, (bg, dc, float(err.max()))
+
+
+@pytest.mark.parametrize("n", [2, 3, 4, 16, 60, 64, 256, 375, 512, 1024, 1500])
+def test_small_parts_beside_large_ones_are_kept(n):
+    """What FP64 additions keep apart: a single complex value at index 0 is the
+    transform's every value; a tiny imaginary background beside a real value
+    there keeps its own relative accuracy."""
+    rng = np.random.default_rng(n)
+    z = np.zeros((9, n), complex)
+    z[:, 0] = rng.normal(size=9) + 1e-9j * rng.normal(size=9)
+    for got in _passes(z):
+        assert (got == z[:, :1]).all()
+    z = 1e-12 * (rng.uniform(-1, 1, (9, n)) + 1j * rng.uniform(-1, 1, (9, n)))
+    z[:, 0] = 1.0
+    ref = np.fft.fft(z.astype(np.clongdouble), axis=1).imag
+    for got in _passes(z):
+        err = np.sqrt(((got.imag.astype(np.longdouble) - ref) ** 2).sum(axis=1) / (ref ** 2).sum(axis=1))
+        assert err.max() <= 1e-15, float(err.max())
