@@ -252,186 +252,198 @@ static bool overlaps_previous(const fft3_plan_s *P, const Launch &L)
 // size, the FP64 roots and then the integer ones.
 static int64_t twiddle_slots(const Schedule &s) { return std::max<int64_t>(16, s.tw_total); }
 
-static int build_launches(fft3_plan_s *P)
+static int build_launch(fft3_plan_s *P, const PassPlan &p, Launch *out)
 {
     const Schedule &s = P->sched;
     const int conj = s.direction == FFT3_INVERSE ? 1 : 0;
-    for (const PassPlan &p : s.passes) {
-        Launch L;
-        L.kind = p.kind;
-        L.src = p.src;
-        L.dst = p.dst;
-        PassArgs &a = L.args;
-        a.g = p.g;
-        a.conj = conj;
-        a.ntiles = p.ntiles;
-        a.tiles_c = p.tiles_c;
-        a.lpt = p.lpt;
-        a.err = P->d_err;
-        // test hooks (options.reserved[0] = slab whose x tiles never signal, plus one;
-        // options.reserved[1] = wait budget in thousands of cycles)
-        a.nosignal_slab = s.opts.reserved[0] > 0 ? (int64_t)s.opts.reserved[0] - 1 : -1;
-        a.wait_budget = s.opts.reserved[1] > 0 ? (long long)s.opts.reserved[1] * 1000LL : 4000000000LL;
-        int64_t base = -1, end = 0;
-        for (int k = 0; k < 3; ++k) {
-            if (p.tw_seg[k] < 0)
-                continue;
-            const TwSeg &sg = s.tw[p.tw_seg[k]];
-            if (base < 0)
-                base = sg.off;
-            end = sg.off + ((int64_t)sg.m.size() + 15) / 16 * 16;
-        }
+    Launch L;
+    L.kind = p.kind;
+    L.src = p.src;
+    L.dst = p.dst;
+    PassArgs &a = L.args;
+    a.g = p.g;
+    a.conj = conj;
+    a.ntiles = p.ntiles;
+    a.tiles_c = p.tiles_c;
+    a.lpt = p.lpt;
+    a.err = P->d_err;
+    // test hooks (options.reserved[0] = slab whose x tiles never signal, plus one;
+    // options.reserved[1] = wait budget in thousands of cycles)
+    a.nosignal_slab = s.opts.reserved[0] > 0 ? (int64_t)s.opts.reserved[0] - 1 : -1;
+    a.wait_budget = s.opts.reserved[1] > 0 ? (long long)s.opts.reserved[1] * 1000LL : 4000000000LL;
+    int64_t base = -1, end = 0;
+    for (int k = 0; k < 3; ++k) {
+        if (p.tw_seg[k] < 0)
+            continue;
+        const TwSeg &sg = s.tw[p.tw_seg[k]];
         if (base < 0)
-            base = 0;
-        a.tw = P->esize == 16 ? (const float2 *)((const double2 *)P->d_tw + base) : P->d_tw + base;
-        if (P->esize == 16)
-            a.tw_fix = (const double2 *)P->d_tw + twiddle_slots(s) + base;
-        a.tw_len = (int)(end - base);
-        if (p.tw_seg[0] >= 0)
-            a.L[0] = to_rt(p.line, (int)(s.tw[p.tw_seg[0]].off - base));
-        if (p.tw_seg[1] >= 0)
-            a.L[1] = to_rt(p.line2, (int)(s.tw[p.tw_seg[1]].off - base));
-        if (p.tw_seg[2] >= 0)
-            a.tw_split_off = (int)(s.tw[p.tw_seg[2]].off - base);
-        a.p = p.p;
-        a.six_step = p.six_step ? 1 : 0;
-        a.split_a = p.split_a;
-        a.split_b = p.split_b;
-        L.probe_g = p.g;
-        L.probe_n = p.line.n;
-        L.smem = p.smem_bytes;
-        L.chunk = p.chunk;
-        L.pair_next = p.pair_next;
-        L.block = dim3(std::max(1, p.threads));
-        const FixedKernels *fk = p.line.fixed >= 0 ? fixed_kernels(p.line.fixed) : nullptr;
-        switch (p.kind) {
-        case PK_J: L.func = fk ? fk->j : nullptr; break;
-        case PK_JROT: L.func = fk ? fk->jrot : nullptr; break;
-        case PK_C: L.func = fk ? (p.lpt == 16 ? fk->c16 : fk->c8) : nullptr; break;
-        case PK_CTMA:
-            L.func = fk ? fk->ctma : nullptr;
-            L.tma = true;
-            break;
-        case PK_G:
-            L.func = p.mixed ? mixed_kernel(p.line.n, p.mixed == 1) : (const void *)&k_pass_g;
-            break;
-        case PK_G64: {
-            const Mixed64Kernels *mk = p.mixed ? mixed64_kernels(p.line.n) : nullptr;
-            L.func = !p.mixed ? (const void *)&k_pass_g64 : mk ? (p.mixed == 1 ? mk->j : mk->c) : nullptr;
-            break;
-        }
-        case PK_J64:
-        case PK_C64: {
-            const Fixed64Kernels *k64 = p.line.fixed >= 0 ? fixed64_kernels(p.line.fixed) : nullptr;
-            L.func = k64 ? (p.kind == PK_J64 ? k64->j : k64->c) : nullptr;
-            break;
-        }
-        case PK_SLAB:
-            L.func = p.mixed ? (const void *)&k_slab_warp : (const void *)&k_slab;
-            L.probe_g = natural_x(s);
-            L.probe_n = s.n0;
-            break;
-        case PK_SLABL2:
-            L.func = fk ? fk->l2 : nullptr;
-            L.reset_counters = true;
-            L.probe_g = natural_x(s);
-            L.probe_n = s.n0;
-            break;
-        case PK_SLABBLK:
-            L.func = fk ? fk->l2blk[p.lpt == 8 ? 1 : 0] : nullptr;
-            L.reset_counters = true;
-            L.slab_map = true;
-            L.probe_g = natural_x(s);
-            L.probe_n = s.n0;
-            break;
-        case PK_VOL:
-            L.func = (const void *)&k_vol;
-            L.cluster = p.p;
-            L.probe_n = p.split_a * p.split_b;
-            break;
-        case PK_VOLC: {
-            int cnt = 0;
-            const VolcKernel *vk = volc_kernels(&cnt);
-            L.func = (p.volc >= 0 && p.volc < cnt) ? vk[p.volc].func : nullptr;
-            L.cluster = p.p;
-            L.probe_n = p.split_a * p.split_b;
-            break;
-        }
-        case PK_CSTREAM: {
-            int cnt = 0;
-            const CStreamKernel *ck = cstream_kernels(&cnt);
-            L.func = (p.cstream >= 0 && p.cstream < cnt)
-                         ? (p.tc_mode < 0 ? ck[p.cstream].func : ck[p.cstream].func_tc[p.tc_mode == 0 ? 0 : 1])
-                         : nullptr;
-            if (L.func && p.tc_mode < 0 && p.src != p.dst && P->elems * 8 >= (int64_t)2 << 30 && ck[p.cstream].func_out)
-                L.func = ck[p.cstream].func_out;
-            L.stream_q = L.func ? ck[p.cstream].q : 0;
-            L.cluster = p.p;
-            break;
-        }
-        case PK_TCX:
-        case PK_TCS:
-            L.func = tc32_kernel(p.kind == PK_TCX ? 0 : 1);
-            L.tc32 = p.kind == PK_TCS ? 2 : 1;
-            break;
-        case PK_JTC:
-            L.func = fk && p.tc_mode >= 0 ? fk->j_tc[p.tc_mode] : nullptr;
-            break;
-        case PK_CTC:
-            L.func = fk && p.tc_mode >= 0 ? fk->c_tc[p.tc_mode] : nullptr;
-            break;
-        case PK_COPY:
-            L.func = (const void *)&k_copy;
-            L.probe_n = 1;
-            break;
-        default: break;
-        }
-        if (!L.func)
-            return fail(FFT3_ERR_UNSUPPORTED_SIZE, "no compiled kernel for this pass");
-        int rc = prepare_func(L.func, L.smem, L.tc32 != 0);
+            base = sg.off;
+        end = sg.off + ((int64_t)sg.m.size() + 15) / 16 * 16;
+    }
+    if (base < 0)
+        base = 0;
+    a.tw = P->esize == 16 ? (const float2 *)((const double2 *)P->d_tw + base) : P->d_tw + base;
+    if (P->esize == 16)
+        a.tw_fix = (const double2 *)P->d_tw + twiddle_slots(s) + base;
+    a.tw_len = (int)(end - base);
+    if (p.tw_seg[0] >= 0)
+        a.L[0] = to_rt(p.line, (int)(s.tw[p.tw_seg[0]].off - base));
+    if (p.tw_seg[1] >= 0)
+        a.L[1] = to_rt(p.line2, (int)(s.tw[p.tw_seg[1]].off - base));
+    if (p.tw_seg[2] >= 0)
+        a.tw_split_off = (int)(s.tw[p.tw_seg[2]].off - base);
+    a.p = p.p;
+    a.six_step = p.six_step ? 1 : 0;
+    a.split_a = p.split_a;
+    a.split_b = p.split_b;
+    L.probe_g = p.g;
+    L.probe_n = p.line.n;
+    L.smem = p.smem_bytes;
+    L.chunk = p.chunk;
+    L.pair_next = p.pair_next;
+    L.unaligned = p.unaligned;
+    L.block = dim3(std::max(1, p.threads));
+    const FixedKernels *fk = p.line.fixed >= 0 ? fixed_kernels(p.line.fixed) : nullptr;
+    switch (p.kind) {
+    case PK_J: L.func = fk ? fk->j : nullptr; break;
+    case PK_JROT: L.func = fk ? fk->jrot : nullptr; break;
+    case PK_C: L.func = fk ? (p.lpt == 16 ? fk->c16 : fk->c8) : nullptr; break;
+    case PK_CTMA:
+        L.func = fk ? fk->ctma : nullptr;
+        L.tma = true;
+        break;
+    case PK_G:
+        L.func = p.mixed ? mixed_kernel(p.line.n, p.mixed == 1) : (const void *)&k_pass_g;
+        break;
+    case PK_G64: {
+        const Mixed64Kernels *mk = p.mixed ? mixed64_kernels(p.line.n) : nullptr;
+        L.func = !p.mixed ? (const void *)&k_pass_g64 : mk ? (p.mixed == 1 ? mk->j : mk->c) : nullptr;
+        break;
+    }
+    case PK_J64:
+    case PK_C64: {
+        const Fixed64Kernels *k64 = p.line.fixed >= 0 ? fixed64_kernels(p.line.fixed) : nullptr;
+        L.func = k64 ? (p.kind == PK_J64 ? k64->j : k64->c) : nullptr;
+        break;
+    }
+    case PK_SLAB:
+        L.func = p.mixed ? (const void *)&k_slab_warp : (const void *)&k_slab;
+        L.probe_g = natural_x(s);
+        L.probe_n = s.n0;
+        break;
+    case PK_SLABL2:
+        L.func = fk ? fk->l2 : nullptr;
+        L.reset_counters = true;
+        L.probe_g = natural_x(s);
+        L.probe_n = s.n0;
+        break;
+    case PK_SLABBLK:
+        L.func = fk ? fk->l2blk[p.lpt == 8 ? 1 : 0] : nullptr;
+        L.reset_counters = true;
+        L.slab_map = true;
+        L.probe_g = natural_x(s);
+        L.probe_n = s.n0;
+        break;
+    case PK_VOL:
+        L.func = (const void *)&k_vol;
+        L.cluster = p.p;
+        L.probe_n = p.split_a * p.split_b;
+        break;
+    case PK_VOLC: {
+        int cnt = 0;
+        const VolcKernel *vk = volc_kernels(&cnt);
+        L.func = (p.volc >= 0 && p.volc < cnt) ? vk[p.volc].func : nullptr;
+        L.cluster = p.p;
+        L.probe_n = p.split_a * p.split_b;
+        break;
+    }
+    case PK_CSTREAM: {
+        int cnt = 0;
+        const CStreamKernel *ck = cstream_kernels(&cnt);
+        L.func = (p.cstream >= 0 && p.cstream < cnt)
+                     ? (p.tc_mode < 0 ? ck[p.cstream].func : ck[p.cstream].func_tc[p.tc_mode == 0 ? 0 : 1])
+                     : nullptr;
+        if (L.func && p.tc_mode < 0 && p.src != p.dst && P->elems * 8 >= (int64_t)2 << 30 && ck[p.cstream].func_out)
+            L.func = ck[p.cstream].func_out;
+        L.stream_q = L.func ? ck[p.cstream].q : 0;
+        L.cluster = p.p;
+        break;
+    }
+    case PK_TCX:
+    case PK_TCS:
+        L.func = tc32_kernel(p.kind == PK_TCX ? 0 : 1);
+        L.tc32 = p.kind == PK_TCS ? 2 : 1;
+        break;
+    case PK_JTC:
+        L.func = fk && p.tc_mode >= 0 ? fk->j_tc[p.tc_mode] : nullptr;
+        break;
+    case PK_CTC:
+        L.func = fk && p.tc_mode >= 0 ? fk->c_tc[p.tc_mode] : nullptr;
+        break;
+    case PK_COPY:
+        L.func = (const void *)&k_copy;
+        L.probe_n = 1;
+        break;
+    default: break;
+    }
+    if (!L.func)
+        return fail(FFT3_ERR_UNSUPPORTED_SIZE, "no compiled kernel for this pass");
+    int rc = prepare_func(L.func, L.smem, L.tc32 != 0);
+    if (rc)
+        return rc;
+    if (p.kind == PK_VOL || p.kind == PK_VOLC || (p.kind == PK_CSTREAM && p.p > 1)) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = p.p;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(p.p * 4);
+        cfg.blockDim = L.block;
+        cfg.dynamicSmemBytes = L.smem;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int ncl = 0;
+        CUDA_TRY(cudaOccupancyMaxActiveClusters(&ncl, L.func, &cfg));
+        if (ncl < 1)
+            return fail(FFT3_ERR_UNSUPPORTED_SIZE, "volumetric cluster does not fit on the GPU");
+        int64_t g = std::min<int64_t>(ncl, p.ntiles);
+        L.grid = dim3((unsigned)(std::max<int64_t>(1, g) * p.p));
+    } else if (p.kind == PK_COPY) {
+        L.grid = dim3((unsigned)std::min<int64_t>(4096, (P->elems * (P->esize / 8) + 255) / 256 + 1));
+        L.block = dim3(256);
+    } else if (p.kind == PK_SLABL2 || p.kind == PK_SLABBLK) {
+        rc = occupancy_grid(L.func, L.block.x, L.smem, 0, P->device, &L.grid);
         if (rc)
             return rc;
-        if (p.kind == PK_VOL || p.kind == PK_VOLC || (p.kind == PK_CSTREAM && p.p > 1)) {
-            cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = p.p;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            cfg.gridDim = dim3(p.p * 4);
-            cfg.blockDim = L.block;
-            cfg.dynamicSmemBytes = L.smem;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            int ncl = 0;
-            CUDA_TRY(cudaOccupancyMaxActiveClusters(&ncl, L.func, &cfg));
-            if (ncl < 1)
-                return fail(FFT3_ERR_UNSUPPORTED_SIZE, "volumetric cluster does not fit on the GPU");
-            int64_t g = std::min<int64_t>(ncl, p.ntiles);
-            L.grid = dim3((unsigned)(std::max<int64_t>(1, g) * p.p));
-        } else if (p.kind == PK_COPY) {
-            L.grid = dim3((unsigned)std::min<int64_t>(4096, (P->elems * (P->esize / 8) + 255) / 256 + 1));
-            L.block = dim3(256);
-        } else if (p.kind == PK_SLABL2 || p.kind == PK_SLABBLK) {
-            rc = occupancy_grid(L.func, L.block.x, L.smem, 0, P->device, &L.grid);
-            if (rc)
-                return rc;
-            P->counters_bytes = std::max(P->counters_bytes,
-                                         (size_t)(1 + p.g.A * p.g.B) * sizeof(int));
-        } else if (L.tc32) {
-            // one block per SM (contiguous lines: each running kTc32Groups streams of tiles)
-            rc = occupancy_grid(L.func, L.block.x, L.smem,
-                                p.kind == PK_TCX ? (p.ntiles + kTc32Groups - 1) / kTc32Groups : p.ntiles,
-                                P->device, &L.grid);
-            if (rc)
-                return rc;
-        } else {
-            rc = occupancy_grid(L.func, L.block.x, L.smem, p.ntiles, P->device, &L.grid);
-            if (rc)
-                return rc;
-        }
-        P->launches.push_back(L);
+        P->counters_bytes = std::max(P->counters_bytes,
+                                     (size_t)(1 + p.g.A * p.g.B) * sizeof(int));
+    } else if (L.tc32) {
+        // one block per SM (contiguous lines: each running kTc32Groups streams of tiles)
+        rc = occupancy_grid(L.func, L.block.x, L.smem,
+                            p.kind == PK_TCX ? (p.ntiles + kTc32Groups - 1) / kTc32Groups : p.ntiles,
+                            P->device, &L.grid);
+        if (rc)
+            return rc;
+    } else {
+        rc = occupancy_grid(L.func, L.block.x, L.smem, p.ntiles, P->device, &L.grid);
+        if (rc)
+            return rc;
     }
+    *out = L;
+    return FFT3_OK;
+}
+
+static int build_launches(fft3_plan_s *P)
+{
+    for (const auto &[from, to] : {std::make_pair(&P->sched.passes, &P->launches), std::make_pair(&P->sched.unaligned, &P->unaligned)})
+        for (const PassPlan &p : *from) {
+            Launch L;
+            int rc = build_launch(P, p, &L);
+            if (rc)
+                return rc;
+            to->push_back(L);
+        }
     bool pair = false;
     for (size_t i = 0; i + 1 < P->launches.size(); ++i)
         pair = pair || (P->launches[i].pair_next && P->launches[i].chunk > 0);
@@ -619,7 +631,7 @@ int fft3_plan_create_ex(fft3_plan *out, int n0, int n1, int n2, int batch, int d
             rc = fail(FFT3_ERR_OOM, "counter allocation failed");
         }
         for (Launch &L : P->launches)
-            L.args.counters = P->d_counters;
+            L.args.counters = P->d_counters; // (stand-ins use none)
     }
     if (rc) {
         free_plan(P);
@@ -641,6 +653,13 @@ int fft3_plan_create(fft3_plan *out, int n0, int n1, int n2, int batch, int dtyp
 static int launch_one(fft3_plan_s *P, const Launch &L, const void *func, PassArgs a, cudaStream_t st,
                       bool after = false)
 {
+    if (L.unaligned >= 0 && ((uintptr_t)a.in & 15)) {
+        const Launch &U = P->unaligned[L.unaligned];
+        PassArgs u = U.args;
+        u.in = a.in;
+        u.out = a.out;
+        return launch_one(P, U, U.func, u, st, after);
+    }
     if (L.reset_counters)
         CUDA_TRY(cudaMemsetAsync(P->d_counters, 0, P->counters_bytes, st));
     cudaLaunchConfig_t cfg = {};

@@ -45,6 +45,7 @@ struct Launch {
     // of a, the next pass's chunk c after this pass's chunk c
     int chunk = 0;
     bool pair_next = false;
+    int unaligned = -1; // index into the plan's `unaligned` launches: this pass for an input aligned to 8 bytes only
     // identity probe of the same pass geometry
     PassGeom probe_g{};
     int probe_n = 1;
@@ -82,6 +83,7 @@ struct fft3_plan_s {
     size_t counters_bytes = 0;
     unsigned *d_err = nullptr;
     std::vector<fft3::Launch> launches;
+    std::vector<fft3::Launch> unaligned; // stand-ins for streamed passes (Launch::unaligned)
     float2 *d_stage_in = nullptr, *d_stage_out = nullptr;
     // pipelined host execution: a second set of staging buffers, the copy and
     // compute streams, and per-set events (input consumed, output produced, output drained)

@@ -591,7 +591,7 @@ static int make_line_pass(Schedule *s, int d, int n, const PassGeom &g, bool rot
     } else if (p.line.fixed >= 0 && !rotate && contig_in && g.ok == 1 && n > 1) {
         p.kind = PK_J;
         p.lpt = lpt_jl(p.line.T);
-    } else if (!rotate && strided_in && n > 1 && (s->opts.tile_lines == 0 || s->opts.tile_lines == kTileStream) &&
+    } else if (!s->no_stream && !rotate && strided_in && n > 1 && (s->opts.tile_lines == 0 || s->opts.tile_lines == kTileStream) &&
                cstream_pick(n, order, g, 1) >= 0) {
         set_cstream(&p, cstream_pick(n, order, g, 1));
     } else if (p.line.fixed >= 0 && !rotate && strided_in && n > 1 && s->opts.tile_lines == kTileTma &&
@@ -753,7 +753,7 @@ static int make_vol_pass(Schedule *s, int d, int n, int p, const PassGeom &g, in
     // the compiled splits of k_volc.cu
     // the blocked six-step comparison schedule runs on the runtime-radix cluster kernel
     const bool six = s->opts.variant == FFT3_VOL_BLOCKED_SIX_STEP;
-    const int ci = !six && p == 2 && s->opts.tile_lines <= kTileStream ? cstream_pick(n, s->opts.radix_order, g, 2)
+    const int ci = !six && !s->no_stream && p == 2 && s->opts.tile_lines <= kTileStream ? cstream_pick(n, s->opts.radix_order, g, 2)
                                                                        : -1;
     if (ci >= 0) {
         PassPlan q;
@@ -1229,7 +1229,8 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
         if (s.opts.variant == FFT3_PPP_NATURAL && (int64_t)n0 * n1 * 8 >= (4ll << 20))
             s.opts.variant = FFT3_PPP_BLOCKED;
     }
-    if (decomp == FFT3_AUTO) {
+    const bool automatic = decomp == FFT3_AUTO;
+    if (automatic) {
         // Fixed default when no cost model is loaded: pencil-pencil-pencil, whose
         // passes are compiled for every length, but slab-pencil up to 1024 values,
         // where a launch less counts (8^3: 5.7 against 7.0 us; 16^3: 8.2 against 7.3).
@@ -1254,18 +1255,42 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
     int64_t N = (int64_t)n0 * n1 * n2;
     int rc = FFT3_OK;
     int cur = BUF_IN;
-    auto add_nat = [&](int d) -> int {
+    // Buffers are asked to be 16-byte aligned, but plans without TMA run on 8 bytes.
+    // A streamed pass that took the place of a kernel with plain loads keeps that
+    // kernel for such an input: `make` plans the pass without streaming.
+    auto keep_unaligned = [&](PassPlan *p, auto make) -> int {
+        if (p->kind != PK_CSTREAM)
+            return FFT3_OK;
+        PassPlan q;
+        s.no_stream = true;
+        const int r = make(&q);
+        s.no_stream = false;
+        if (!r) {
+            p->unaligned = (int)s.unaligned.size();
+            s.unaligned.push_back(q);
+        }
+        return r;
+    };
+    auto add_nat = [&](int d, bool unaligned = false) -> int {
         if (ns[d] == 1)
             return FFT3_OK;
         PassPlan p;
-        int r = make_line_pass(&s, d, ns[d], geom_natural(d, n0, n1, n2, batch), false, cur, BUF_OUT,
-                               &p, err);
+        const int from = cur;
+        auto make = [&](PassPlan *q) {
+            return make_line_pass(&s, d, ns[d], geom_natural(d, n0, n1, n2, batch), false, from, BUF_OUT, q, err);
+        };
+        int r = make(&p);
+        if (!r && unaligned)
+            r = keep_unaligned(&p, make);
         if (r)
             return r;
         s.passes.push_back(p);
         cur = BUF_OUT;
         return FFT3_OK;
     };
+    // slabs that fit one block's shared memory: their y lines were no streamed pass
+    // of their own under FFT3_AUTO and the slab-pencil default before they became one
+    const bool slab_fits = slab_smem(n0, n1, 2 * tw_slots_h(n0) + 2 * tw_slots_h(n1)) <= kSmemLimit;
     // Blocked intermediate (FFT3_PPP_BLOCKED): x pass natural, y pass from `out`
     // into the workspace laid out as [x/16][z][y][x%16] (a 16-column tile of y
     // lines is one contiguous block), z pass from the workspace back to `out`.
@@ -1418,12 +1443,11 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
         s.need_ws = true;
     } else if (decomp == FFT3_PENCIL3) {
         for (int d = 0; d < 3 && !rc; ++d)
-            rc = add_nat(d);
+            rc = add_nat(d, automatic && d == 1 && slab_fits);
     } else if (decomp == FFT3_SLAB_PENCIL) {
         bool z_done = false;
         int mode = s.opts.slab_mode;
-        int twl = 2 * tw_slots_h(n0) + 2 * tw_slots_h(n1);
-        bool fits_smem = slab_smem(n0, n1, twl) <= kSmemLimit;
+        const bool fits_smem = slab_fits;
         if (mode == 0)
             // The L2-resident slab kernel measured slower than x and y passes (256^2 to
             // 1024^2), and so does the shared-memory one, whose radix lists are data, once
@@ -1483,7 +1507,7 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
             // unfused slab stage: x lines then y lines as two passes
             rc = add_nat(0);
             if (!rc)
-                rc = add_nat(1);
+                rc = add_nat(1, s.opts.slab_mode == 0 && slab_fits);
         }
         if (!rc && !z_done)
             rc = add_nat(2);
@@ -1521,7 +1545,10 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
             if (p == 1) {
                 rc = make_line_pass(&s, d, ns[d], g, false, cur, BUF_OUT, &q, err);
             } else {
-                rc = make_vol_pass(&s, d, ns[d], p, g, cur, BUF_OUT, &q, err);
+                auto make = [&](PassPlan *v) { return make_vol_pass(&s, d, ns[d], p, g, cur, BUF_OUT, v, err); };
+                rc = make(&q);
+                if (!rc && ns[d] < 512) // k_volc and k_vol take these lengths with plain loads
+                    rc = keep_unaligned(&q, make);
             }
             if (rc)
                 return rc;

@@ -72,6 +72,7 @@ struct PassPlan {
     int chunk = 0;              // slabs per chunk of a two-stream pipelined slab stage (0 = one launch)
     bool pair_next = false;     // this pass and the next run chunk-interleaved on two streams
     bool six_step = false;      // PK_VOL: blocked ownership, three exchanges (Section 2.2)
+    int unaligned = -1;         // index into Schedule::unaligned: the pass for an input that TMA cannot read
 };
 
 struct Schedule {
@@ -79,6 +80,8 @@ struct Schedule {
     int dtype = FFT3_C64_FP32, decomp = FFT3_PENCIL3, direction = FFT3_FORWARD;
     fft3_options opts{};
     std::vector<PassPlan> passes;
+    std::vector<PassPlan> unaligned; // stand-ins of streamed passes for inputs aligned to 8 bytes only
+    bool no_stream = false;          // planning such a stand-in
     std::vector<TwSeg> tw;
     int64_t tw_total = 0;
     bool need_ws = false;
