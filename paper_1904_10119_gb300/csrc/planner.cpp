@@ -1229,12 +1229,17 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
         if (s.opts.variant == FFT3_PPP_NATURAL && (int64_t)n0 * n1 * 8 >= (4ll << 20))
             s.opts.variant = FFT3_PPP_BLOCKED;
     }
+    // whether a slab fits one block's shared memory (k_slab)
+    const bool slab_fits = slab_smem(n0, n1, 2 * tw_slots_h(n0) + 2 * tw_slots_h(n1)) <= kSmemLimit;
     const bool automatic = decomp == FFT3_AUTO;
     if (automatic) {
         // Fixed default when no cost model is loaded: pencil-pencil-pencil, whose
         // passes are compiled for every length, but slab-pencil up to 1024 values,
         // where a launch less counts (8^3: 5.7 against 7.0 us; 16^3: 8.2 against 7.3).
-        decomp = (int64_t)n0 * n1 * n2 * batch <= 1024 ? FFT3_SLAB_PENCIL : FFT3_PENCIL3;
+        // A caller that names a slab mode gets the slab schedule wherever a slab fits one
+        // block's shared memory, and the mode's refusals.
+        decomp = (int64_t)n0 * n1 * n2 * batch <= 1024 || (s.opts.slab_mode != 0 && slab_fits) ? FFT3_SLAB_PENCIL
+                                                                                               : FFT3_PENCIL3;
         // and with the blocked intermediate when it applies, from 256 MiB on, unless the
         // natural z lines are 512 points at 2 to 4 MiB (natural / blocked, us: 512 x 512 x
         // 512 1026 / 1064, 256 x 1024 x 512 1047 / 1060; but 240 x 512 x 512 552 / 481,
@@ -1288,9 +1293,6 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
         cur = BUF_OUT;
         return FFT3_OK;
     };
-    // slabs that fit one block's shared memory: their y lines were no streamed pass
-    // of their own under FFT3_AUTO and the slab-pencil default before they became one
-    const bool slab_fits = slab_smem(n0, n1, 2 * tw_slots_h(n0) + 2 * tw_slots_h(n1)) <= kSmemLimit;
     // Blocked intermediate (FFT3_PPP_BLOCKED): x pass natural, y pass from `out`
     // into the workspace laid out as [x/16][z][y][x%16] (a 16-column tile of y
     // lines is one contiguous block), z pass from the workspace back to `out`.
@@ -1443,7 +1445,7 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
         s.need_ws = true;
     } else if (decomp == FFT3_PENCIL3) {
         for (int d = 0; d < 3 && !rc; ++d)
-            rc = add_nat(d, automatic && d == 1 && slab_fits);
+            rc = add_nat(d, automatic && d == 1 && slab_fits); // once lines of a slab kernel
     } else if (decomp == FFT3_SLAB_PENCIL) {
         bool z_done = false;
         int mode = s.opts.slab_mode;

@@ -222,6 +222,18 @@ def test_null_arguments(lib):
     assert lib.fft3_plan_destroy(None) == -1
 
 
+@pytest.mark.parametrize("mode", range(1, 6))
+@pytest.mark.parametrize("shape", [(32, 32, 32), (16, 512, 16), (60, 45, 50)])
+def test_automatic_plan_with_a_slab_mode_is_the_slab_schedule(shape, mode):
+    """FFT3_AUTO honours a named slab mode where a slab fits shared memory, refusals included."""
+    def plan(decomposition):
+        try:
+            return fft3.fft3_plan_schedule(*shape, 1, 0, decomposition, -1, fft3.make_options(slab_mode=mode))["passes"]
+        except fft3.Fft3Error as e:
+            return str(e)
+    assert plan(fft3.FFT3_AUTO) == plan(fft3.FFT3_SLAB_PENCIL)
+
+
 def test_volumetric_automatic_mesh_and_compiled_splits():
     # automatic mesh: the strided 1024-point lines split over a cluster pair,
     # each block streaming half of the decimated sub-lines
