@@ -621,6 +621,12 @@ int fft3_plan_create_ex(fft3_plan *out, int n0, int n1, int n2, int batch, int d
         e = cudaMalloc(&P->d_ws, P->ws_bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
+            // FFT3_AUTO's blocked intermediate is a choice for speed: without room for it, the natural order
+            if (decomposition == FFT3_AUTO && P->sched.opts.variant == FFT3_PPP_BLOCKED &&
+                !(opts && (opts->variant == FFT3_PPP_BLOCKED || opts->layout != FFT3_LAYOUT_NATURAL))) {
+                free_plan(P);
+                return fft3_plan_create_ex(out, n0, n1, n2, batch, dtype, FFT3_PENCIL3, direction, opts);
+            }
             rc = fail(FFT3_ERR_OOM, "workspace allocation failed");
         }
     }
