@@ -671,8 +671,10 @@ int fft3_mlp_train(fft3_mlp m, const float *h_X, const float *h_y, int n, int ep
         cudaFree(dyb);
         cudaFree(didx);
     };
+    // gathered minibatches and activations: the layer-by-layer kernels alone need them
+    const bool layers = !m->grad_ws;
     if (cudaMalloc(&dX, (size_t)n * F * 4) || cudaMalloc(&dy, (size_t)n * 4) ||
-        cudaMalloc(&dXb, (size_t)batch * F * 4) || cudaMalloc(&dyb, (size_t)batch * 4) ||
+        (layers && (cudaMalloc(&dXb, (size_t)batch * F * 4) || cudaMalloc(&dyb, (size_t)batch * 4))) ||
         cudaMalloc(&didx, (size_t)n * 4)) {
         cudaGetLastError();
         cleanup();
@@ -680,7 +682,7 @@ int fft3_mlp_train(fft3_mlp m, const float *h_X, const float *h_y, int n, int ep
     }
     cudaMemcpy(dX, h_X, (size_t)n * F * 4, cudaMemcpyHostToDevice);
     cudaMemcpy(dy, h_y, (size_t)n * 4, cudaMemcpyHostToDevice);
-    int rc = mlp_reserve(m, std::max(batch, n));
+    int rc = layers ? mlp_reserve(m, n) : FFT3_OK;
     std::vector<int> perm(n);
     for (int i = 0; i < n; ++i)
         perm[i] = i;

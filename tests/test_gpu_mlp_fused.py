@@ -39,3 +39,16 @@ def test_gradient_matches_fp64_oracle_and_repeats(F, H, B):
     assert np.linalg.norm(got - ref) <= 2e-6 * np.linalg.norm(ref)
     assert abs(losses[0].item() - oracle.mse_loss(pred, y)) <= 2e-6 * oracle.mse_loss(pred, y)
     m.close()
+
+
+def test_training_keeps_no_activations():
+    """The one-launch gradient needs no activations: training leaves none with the handle."""
+    n, F = 1 << 18, 8
+    rng = np.random.default_rng(0)
+    X, y = rng.normal(size=(n, F)).astype(np.float32), rng.normal(size=n).astype(np.float32)
+    m = fft3.Mlp(F, 64, seed=1)
+    m.train(X[:256], y[:256], epochs=1, batch=128, lr=1e-3, seed=1)  # loads the kernels
+    free = torch.cuda.mem_get_info()[0]
+    m.train(X, y, epochs=1, batch=n, lr=1e-3, seed=1)
+    assert free - torch.cuda.mem_get_info()[0] < 64 << 20  # activations of all samples: 6 x 64 MiB
+    m.close()
