@@ -457,10 +457,10 @@ int fft3_execute_noalloc(int n0, int n1, int n2, int batch, int direction, const
  * choice of decomposition to the user; Section 4.3 shows no single one wins) */
 
 /* Times one plan: creates it, allocates two scratch arrays of the problem's
- * size, runs two untimed executions and `reps` timed ones (CUDA events on the
- * legacy default stream), destroys everything, and writes the mean ms of one
- * execution to *ms (for a plan whose `reps` executions take less than 0.1 ms:
- * the smallest of three means over about 0.1 ms each). */
+ * size, runs a few untimed executions and three timed groups (CUDA events on the
+ * legacy default stream) of a third of `reps` executions or as many as take about
+ * 0.1 ms, destroys everything, and writes the smallest group's mean ms of one
+ * execution to *ms. */
 int fft3_time_plan(int n0, int n1, int n2, int batch, int dtype, int decomposition, int direction,
                    const fft3_options *opts, int reps, float *ms);
 

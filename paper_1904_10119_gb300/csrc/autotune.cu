@@ -45,10 +45,10 @@ struct Scratch {
     }
 };
 
-// Mean ms of `reps` executions between two events; for plans so short that
-// launches and event resolution scatter it (reps executions under 0.1 ms:
-// repeated timings of one plan differed by 5%), the smallest of three such
-// means, over as many executions as take about 0.1 ms.
+// The smallest of three means, each over a third of `reps` executions and over as
+// many as take about 0.1 ms between two events (launches and event resolution
+// scatter shorter ones: repeated timings of one plan differed by 5%).  The same
+// statistic for every plan, so that the candidates of one tuning call compare.
 int time_plan(fft3_plan p, const void *in, void *out, int reps, float *ms)
 {
     cudaEvent_t e0, e1;
@@ -58,7 +58,7 @@ int time_plan(fft3_plan p, const void *in, void *out, int reps, float *ms)
     if (!rc)
         rc = fft3_plan_execute(p, in, out, nullptr);
     cudaError_t e = cudaSuccess;
-    int n = std::max(1, reps);
+    int n = std::max(1, (reps + 2) / 3);
     float best = 0.f;
     for (int group = 0; group < 4 && !rc && e == cudaSuccess; ++group) {
         cudaEventRecord(e0, nullptr);
@@ -70,11 +70,8 @@ int time_plan(fft3_plan p, const void *in, void *out, int reps, float *ms)
         if (!rc && e == cudaSuccess)
             cudaEventElapsedTime(&t, e0, e1);
         best = group <= 1 ? t / n : std::min(best, t / n); // group 0 only tells how many executions to time
-        if (group == 0) {
-            if (t >= 0.1f)
-                break;
+        if (group == 0)
             n = std::max(n, (int)(0.1f / std::max(t / n, 1e-3f)));
-        }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
