@@ -67,8 +67,9 @@ enum fft3_decomp {
     FFT3_VOLUMETRIC = 2,  /* every 1D DFT split over p cooperating blocks (Section 3.2) */
     FFT3_AUTO = 3         /* the planner's fixed rule: pencil-pencil-pencil, with the blocked intermediate
                              where it applies (and its array-sized workspace can be allocated), or
-                             slab-pencil up to 1024 values and wherever options name a slab mode
-                             for slabs that fit one block's shared memory; fft3_autotune and the
+                             slab-pencil up to 1024 values (2^15 in small slabs of warp-register
+                             lengths) and wherever options name a slab mode for slabs that fit
+                             one block's shared memory; fft3_autotune and the
                              learned chooser pick by measurement */
 };
 

@@ -835,6 +835,17 @@ static bool warp_line(int n, LineChoice *lc)
     return false;
 }
 
+// Whether the slab pass runs k_slab_warp: both sides of a compiled warp-register
+// length under the default radix order, but not for more small slabs than
+// multiprocessors, which leave its 256 threads idle (16 x 16: 1024 slabs 12.4 us,
+// with k_slab 10.3; 16 slabs 6.4, with k_slab 7.3).
+constexpr int kSms = 152; // GB300's multiprocessors (plans are made without a device, too)
+static bool slab_warp(int n0, int n1, int64_t slabs, int radix_order)
+{
+    LineChoice lc;
+    return radix_order == 0 && ((int64_t)n0 * n1 >= 384 || slabs <= kSms) && warp_line(n0, &lc) && warp_line(n1, &lc);
+}
+
 static int make_slab_pass(Schedule *s, int n0, int n1, int64_t n2, int64_t batch, PassPlan *out,
                           std::string *err)
 {
@@ -850,11 +861,9 @@ static int make_slab_pass(Schedule *s, int n0, int n1, int64_t n2, int64_t batch
     q.g.ij = 1; q.g.ic = 0; q.g.ia = (int64_t)n0 * n1; q.g.ib = N;
     q.g.ok = 1; q.g.oc = 0; q.g.oa = q.g.ia; q.g.ob = N;
     q.lpt = 1;
-    // Both sides of a compiled warp-register length: k_slab_warp (default radix order), but
-    // not for more small slabs than multiprocessors, which leave its 256 threads idle
-    // (16 x 16: 1024 slabs 12.4 us, with k_slab 10.3; 16 slabs 6.4, with k_slab 7.3).
-    const bool busy = (int64_t)n0 * n1 >= 384 || n2 * batch <= 152;
-    if (busy && s->opts.radix_order == 0 && warp_line(n0, &q.line) && warp_line(n1, &q.line2)) {
+    if (slab_warp(n0, n1, n2 * batch, s->opts.radix_order)) {
+        warp_line(n0, &q.line);
+        warp_line(n1, &q.line2);
         q.mixed = 1;
         q.smem_bytes = n1 * (n0 | 1) * 8;
         q.threads = 256;
@@ -1233,15 +1242,21 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
     const bool slab_fits = slab_smem(n0, n1, 2 * tw_slots_h(n0) + 2 * tw_slots_h(n1)) <= kSmemLimit;
     const bool automatic = decomp == FFT3_AUTO;
     if (automatic) {
-        // Fixed default when no cost model is loaded: pencil-pencil-pencil, whose
-        // passes are compiled for every length, but slab-pencil up to 1024 values,
-        // where a launch less counts (8^3: 5.7 against 7.0 us; 16^3: 8.2 against 7.3).
+        // Fixed default when no cost model is loaded: pencil-pencil-pencil, but slab-pencil
+        // where a launch less counts for more than its kernel's slower lines (slab-pencil /
+        // passes, us): up to 1024 values (8^3 5.3 / 7.0, 8 x 8 x 16 5.3 / 7.2; 10^3, k_slab,
+        // 7.2 / 7.1), and up to 2^15 in slabs of at most 1024 where k_slab_warp runs (16^3 6.2 /
+        // 8.0, 24^3 7.1 / 8.2, 32 x 32 x 8 6.2 / 8.0, 32^3 6.5 / 8.2, 8 x 16 x 128 6.2 / 8.5; but
+        // 32 x 32 x 64 and 40 x 32 x 24 8.2 / 8.2, 80 x 48 x 8 10.2 / 8.1, 96 x 96 x 3 12.3 /
+        // 8.4; k_slab: 12^3 7.2 / 7.4, 20^3 8.2 / 7.8, 30^3 10.3 / 8.4).
         // A caller that names a slab mode gets the slab schedule wherever a slab fits one
         // block's shared memory, and the mode's refusals.
-        decomp = (int64_t)n0 * n1 * n2 * batch <= 1024 || (s.opts.slab_mode != 0 && slab_fits) ? FFT3_SLAB_PENCIL
-                                                                                               : FFT3_PENCIL3;
-        // and with the blocked intermediate when it applies, from 256 MiB on, unless the
-        // natural z lines are 512 points at 2 to 4 MiB (natural / blocked, us: 512 x 512 x
+        const int64_t values = (int64_t)n0 * n1 * n2 * batch;
+        const bool small = values <= 1024 || (values <= (1 << 15) && n0 * n1 <= 1024 &&
+                                              slab_warp(n0, n1, (int64_t)n2 * batch, s.opts.radix_order));
+        decomp = small || (s.opts.slab_mode != 0 && slab_fits) ? FFT3_SLAB_PENCIL : FFT3_PENCIL3;
+        // and with the blocked intermediate when it applies (z lines of 512 and 1024 points),
+        // from 256 MiB on, unless 512-point z lines lie 2 to 4 MiB apart (natural / blocked, us: 512 x 512 x
         // 512 1026 / 1064, 256 x 1024 x 512 1047 / 1060; but 240 x 512 x 512 552 / 481,
         // 480 x 512 x 512 1002 / 986, 512 x 512 x 1024 2136 / 2054, 1024 x 1024 x 512
         // 4430 / 4133; below 256 MiB within 1%, or the natural order ahead by up to 5%)

@@ -222,6 +222,17 @@ def test_null_arguments(lib):
     assert lib.fft3_plan_destroy(None) == -1
 
 
+@pytest.mark.parametrize("shape,batch,slab", [
+    ((16, 16, 16), 1, True), ((32, 32, 32), 1, True), ((16, 16, 16), 8, True), ((8, 16, 128), 1, True), ((10, 10, 10), 1, True),
+    ((80, 48, 8), 1, False), ((32, 32, 36), 1, False), ((16, 16, 64), 4, False), ((20, 20, 20), 1, False), ((64, 64, 64), 1, False)])
+def test_automatic_plan_of_small_boxes(shape, batch, slab):
+    """Slab-pencil up to 1024 values, and up to 2^15 in slabs of at most 1024 that run compiled warp-register lines."""
+    s = fft3.fft3_plan_schedule(*shape, batch, 0, fft3.FFT3_AUTO, -1)
+    first = s["passes"][0]
+    assert (first["kind"] == "slab_smem") == slab
+    assert not slab or first.get("compiled") or shape[0] * shape[1] * shape[2] * batch <= 1024
+
+
 @pytest.mark.parametrize("mode", range(1, 6))
 @pytest.mark.parametrize("shape", [(32, 32, 32), (16, 512, 16), (60, 45, 50)])
 def test_automatic_plan_with_a_slab_mode_is_the_slab_schedule(shape, mode):
