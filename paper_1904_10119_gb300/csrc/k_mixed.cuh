@@ -29,6 +29,7 @@ struct SmemLineMixed { // position p at p + (p >> SH), SH = 0: p
 template <int N, int T, int LPT, int MB, int SH, int PITCH, class Rad>
 __global__ void __launch_bounds__(T *LPT, MB) k_mixed_j(PassArgs a)
 {
+    static_assert(MB <= 32, "an SM holds 32 blocks; a larger bound is ignored");
     extern __shared__ float2 smem[];
     float2 *tw = smem;
     float2 *buf = smem + tw_slots(a.tw_len);
@@ -52,6 +53,7 @@ __global__ void __launch_bounds__(T *LPT, MB) k_mixed_j(PassArgs a)
 template <int N, int T, int LPT, int MB, class Rad>
 __global__ void __launch_bounds__(T *LPT, MB) k_mixed_c(PassArgs a)
 {
+    static_assert(MB <= 32, "an SM holds 32 blocks; a larger bound is ignored");
     extern __shared__ float2 smem[];
     float2 *tw = smem;
     float2 *buf = smem + tw_slots(a.tw_len);

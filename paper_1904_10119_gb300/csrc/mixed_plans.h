@@ -11,8 +11,9 @@
 // of the radices 2, 3, 4, 5, 6, 8, 9, 10, 12, 15 and 16 with product N in every
 // order that starts with a large one, T that leaves few of the N / R butterflies
 // of a stage without a thread (at most 30 values per thread), blocks of 512,
-// 768 or 1024 threads per SM, the six best by instructions per value and bank
-// conflicts; SH and PITCH are those with the fewest conflicts over all stages,
+// 768 or 1024 threads per SM as far as 32 resident blocks allow (one thread a
+// column makes blocks of 16: half a warp each, 512 threads per SM), the six best
+// by instructions per value and bank conflicts; SH and PITCH are those with the fewest conflicts over all stages,
 // counted from the addresses of each warp.  The padding of the power-of-two
 // plans (SH = 4) costs odd radices 3 to 5 times the accesses: 375 points ran
 // at 2.8 TB/s with it, at 4.9 without.  Rates of the rows below on 268 MB (one
@@ -35,7 +36,7 @@
     X(900, 60, 4, 4, 0, 908, 15, 4, 15)
 
 #define FFT3_MIXED_C_A(X)                                                               \
-    X(3, 1, 16, 32, 3) X(10, 1, 16, 64, 10) X(20, 2, 16, 24, 10, 2)                     \
+    X(3, 1, 16, 32, 3) X(10, 1, 16, 32, 10) X(20, 2, 16, 24, 10, 2)                     \
     X(30, 2, 16, 24, 15, 2) X(48, 4, 16, 12, 12, 4) X(72, 6, 16, 8, 12, 6)              \
     X(90, 10, 16, 7, 10, 9) X(120, 12, 16, 6, 12, 10) X(150, 15, 16, 5, 15, 10)         \
     X(192, 16, 16, 4, 16, 12) X(240, 18, 16, 4, 16, 15) X(288, 24, 16, 3, 12, 6, 4)     \
@@ -56,7 +57,7 @@
     X(960, 64, 4, 3, 4, 1019, 16, 15, 4)
 
 #define FFT3_MIXED_C_B(X)                                                                   \
-    X(5, 1, 16, 64, 5) X(12, 1, 16, 32, 12) X(24, 2, 16, 24, 12, 2)                         \
+    X(5, 1, 16, 32, 5) X(12, 1, 16, 32, 12) X(24, 2, 16, 24, 12, 2)                         \
     X(36, 3, 16, 16, 12, 3) X(50, 5, 16, 13, 10, 5) X(75, 5, 16, 10, 15, 5)                 \
     X(96, 4, 16, 12, 12, 8) X(125, 5, 16, 7, 5, 5, 5) X(160, 16, 16, 4, 16, 10)             \
     X(200, 10, 16, 5, 10, 5, 4) X(243, 9, 16, 4, 9, 9, 3) X(300, 10, 16, 4, 10, 6, 5)       \
@@ -77,7 +78,7 @@
     X(972, 54, 4, 4, 0, 982, 9, 12, 9)
 
 #define FFT3_MIXED_C_C(X)                                                               \
-    X(6, 1, 16, 48, 6) X(15, 1, 16, 48, 15) X(25, 1, 16, 32, 5, 5)                      \
+    X(6, 1, 16, 32, 6) X(15, 1, 16, 32, 15) X(25, 1, 16, 32, 5, 5)                      \
     X(40, 2, 16, 16, 10, 4) X(54, 6, 16, 11, 9, 6) X(80, 10, 16, 7, 10, 8)              \
     X(100, 10, 16, 7, 10, 10) X(135, 9, 16, 6, 15, 3, 3) X(162, 9, 16, 6, 9, 6, 3)      \
     X(216, 18, 16, 4, 6, 6, 6) X(250, 25, 16, 3, 10, 5, 5) X(320, 40, 8, 4, 10, 8, 4)   \
@@ -98,7 +99,7 @@
     X(1000, 50, 5, 3, 0, 1001, 10, 10, 10)
 
 #define FFT3_MIXED_C_D(X)                                                                 \
-    X(9, 1, 16, 48, 9) X(18, 2, 16, 24, 9, 2) X(27, 3, 16, 22, 9, 3)                      \
+    X(9, 1, 16, 32, 9) X(18, 2, 16, 24, 9, 2) X(27, 3, 16, 22, 9, 3)                      \
     X(45, 3, 16, 16, 15, 3) X(60, 6, 16, 11, 12, 5) X(81, 9, 16, 8, 9, 9)                 \
     X(108, 12, 16, 6, 12, 9) X(144, 14, 16, 5, 12, 12) X(180, 15, 16, 5, 15, 12)          \
     X(225, 17, 16, 4, 15, 15) X(270, 30, 16, 3, 10, 9, 3) X(324, 18, 16, 3, 9, 6, 6)      \

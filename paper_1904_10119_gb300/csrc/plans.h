@@ -174,8 +174,8 @@ const FixedKernels *fixed_kernels(int id);
 // complex128 passes of a fixed plan (k_pass64.cu): contiguous lines, lpt_j64(T)
 // lines per tile; strided lines, kLpt64Strided columns per tile (0 if not compiled)
 constexpr int kLpt64Strided = 8;
-// Blocks of 128 threads (contiguous) and of at least 64 (strided: `groups64` tiles
-// side by side): the kernels' phases (loads, conversions, butterflies, rounding)
+// Blocks of 128 threads (contiguous) and of 64, or down to 40 where T divides 64
+// badly (strided: `groups64` tiles side by side): the kernels' phases (loads, conversions, butterflies, rounding)
 // use different pipes, and small blocks keep more phases in flight at once.
 // 256^3: contiguous blocks of 256 / 128 / 64 threads 199 / 183 / 187 us, strided
 // 207 (256) / 195 (128); 16-point columns 40 us with 8 threads a block, 18 with 64.
