@@ -402,9 +402,13 @@ class Plan:
         want = torch.complex128 if self.dtype == FFT3_C128_FP64 else torch.complex64
         assert x.is_cuda and out.is_cuda and x.dtype == want and out.dtype == want
         assert x.is_contiguous() and out.is_contiguous()
-        # the current stream's handle without a Stream object around it: a transform of
-        # a few microseconds is bound by this call
-        s = stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        if stream is None:
+            # the current stream's handle without a Stream object around it, where torch
+            # has that (not a public name): a transform of a few microseconds is bound by this call
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            s = raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
+        else:
+            s = stream.cuda_stream
         fft3_plan_execute(self.handle, x.data_ptr(), out.data_ptr(), s)
 
     def describe(self) -> dict:
