@@ -622,9 +622,9 @@ def dist_table(fft3, torch, n, hbm, ranks=(2, 4, 8), reps=10):
 
 
 def c128_table(fft3, synth, torch, sizes=(256, 512, 1024), reps=5):
-    """complex128 (FP64 butterflies and twiddles) forward ms of n^3, out of
-    place, CUDA events over `reps` back-to-back executions; GFLOP/s in the
-    5 N log2 N convention (the path is bound by FP64 arithmetic)."""
+    """complex128 (64-bit block fixed point inside a line) forward ms of n^3, out
+    of place, CUDA events over `reps` back-to-back executions; GFLOP/s in the
+    5 N log2 N convention."""
     import math
     table = {}
     st = torch.cuda.current_stream()

@@ -126,7 +126,9 @@ enum fft3_vol_variant {
 /* Optional planner controls.  Zero-initialise and set what you need. */
 typedef struct fft3_options {
     int variant;      /* fft3_ppp_variant for FFT3_PENCIL3, fft3_vol_variant for FFT3_VOLUMETRIC */
-    int radix_order;  /* index into the candidate radix orders of each line length (0 = default) */
+    int radix_order;  /* index into the candidate radix orders of each line length (0 = default; the
+                         streamed passes have candidates of their own, and contiguous complex64 lines
+                         of 16, 64 and 128 points count their first two in the opposite order) */
     int tile_lines;   /* strided passes: 0 = default (the streamed kernel where one is
                          compiled for the line length, else 16 lines per tile);
                          8 or 16 = lines per tile of the plain strided kernel;

@@ -9,7 +9,9 @@
 // instructions per value at no more than 16 values a thread (128 registers), then
 // the stage order, SH and PITCH with the fewest bank conflicts of 16-byte
 // accesses.  The runtime lists (16, 8, 4, 2, 5, 3) of the other lengths take a
-// quarter of the rate: 240^3 in 1810 us against 644.
+// third of the rate: 240^3 in 1810 us against 656.  The list ends at 512 points;
+// longer mixed lengths (540 to 1000 points) keep the runtime lists, no compiled plan
+// of theirs was measured.
 #pragma once
 
 #define FFT3_MIXED64_A(X)                                            \

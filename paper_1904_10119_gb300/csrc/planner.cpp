@@ -1223,9 +1223,9 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
         return FFT3_OK;
     }
     if (dtype == FFT3_C128_FP64) {
-        // complex128 runs every line transform as one pass of the runtime-radix
-        // complex128 kernel: pencil-pencil-pencil in natural order (the slab-pencil
-        // and automatic choices lower to the same three passes)
+        // complex128: pencil-pencil-pencil in natural order, each line transform one pass
+        // (compiled for the fixed and mixed plans, else of the runtime-radix kernel); the
+        // slab-pencil and automatic choices lower to the same three passes
         if (decomp == FFT3_VOLUMETRIC || s.opts.variant != FFT3_PPP_NATURAL ||
             s.opts.layout != FFT3_LAYOUT_NATURAL) {
             *err = "complex128 runs the natural pencil-pencil-pencil schedule";
@@ -1467,9 +1467,11 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
         const bool fits_smem = slab_fits;
         if (mode == 0)
             // The L2-resident slab kernel measured slower than x and y passes (256^2 to
-            // 1024^2), and so does the shared-memory one, whose radix lists are data, once
-            // its values count for more than the launch it saves (slab / passes, us: 96 x 96
-            // x 1000 211 / 82, 54 x 18 x 576 x 4 66 / 25, 16 x 16 x 16 x 1000 57 / 37).
+            // 1024^2).  The shared-memory ones are what slab-pencil asks for and keep small
+            // arrays, where they lead or cost a few us (slab / passes, us: 16^3 6.2 / 7.5,
+            // 48^3 8.2 / 8.2, 64^3 10.3 / 8.3, 60 x 45 x 50 14.4 / 10.2); beyond 2^18 values
+            // they cost a multiple (96 x 96 x 1000 211 / 82, 54 x 18 x 576 x 4 66 / 25, 16^3
+            // x 1000 57 / 37).
             mode = fits_smem && N * batch <= (1 << 18) ? 1 : 3;
         PassPlan p;
         if (mode == 1 && fits_smem) {

@@ -1,5 +1,5 @@
-"""complex128 path (the paper's own precision, Section 4: complex double):
-FP64 butterflies and FP64 twiddles against the FP64 oracle, through the C ABI."""
+"""complex128 path (the paper's own precision, Section 4: complex double) against
+the FP64 oracle, through the C ABI."""
 import numpy as np
 import pytest
 import torch
@@ -37,8 +37,8 @@ def _run(shape, batch, direction, seed, decomposition=fft3.FFT3_PENCIL3, x=None)
     ((256, 256, 8), 1, fft3.FFT3_FORWARD), ((5, 1, 1), 2, fft3.FFT3_FORWARD), ((512, 64, 32), 1, fft3.FFT3_INVERSE),
     ((64, 1024, 3), 1, fft3.FFT3_FORWARD), ((24, 16, 1024), 1, fft3.FFT3_INVERSE)])
 def test_c128_parity(shape, batch, direction):
-    """FP64 passes: the compiled ones (contiguous and strided lines of a fixed
-    plan's length) and the runtime-radix one, ragged tiles included."""
+    """The compiled passes (contiguous and strided lines of a fixed or mixed plan's
+    length) and the runtime-radix one, ragged tiles included."""
     x, got, _ = _run(shape, batch, direction, seed=sum(shape) + batch)
     ref = oracle.fft3(x.ravel(), *shape, batch, sign=direction)
     assert np.all(np.isfinite(got))
