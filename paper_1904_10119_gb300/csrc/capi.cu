@@ -492,30 +492,27 @@ static int generate_twiddles(fft3_plan_s *P)
     const int64_t total = twiddle_slots(s) * (fp64 ? 2 : 1);
     CUDA_TRY(cudaMalloc(&P->d_tw, total * P->esize));
     CUDA_TRY(cudaMemset(P->d_tw, 0, total * P->esize));
-    size_t maxm = 1;
+    // every table's exponents in one upload, each at its table's offset
+    std::vector<int64_t> m(std::max<int64_t>(1, s.tw_total));
     for (const TwSeg &sg : s.tw)
-        maxm = std::max(maxm, sg.m.size());
+        std::copy(sg.m.begin(), sg.m.end(), m.begin() + sg.off);
     int64_t *d_m = nullptr;
-    CUDA_TRY(cudaMalloc(&d_m, maxm * sizeof(int64_t)));
+    CUDA_TRY(cudaMalloc(&d_m, m.size() * sizeof(int64_t)));
+    cudaError_t e = cudaMemcpy(d_m, m.data(), m.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
     for (const TwSeg &sg : s.tw) {
-        cudaError_t e = cudaMemcpy(d_m, sg.m.data(), sg.m.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) {
-            int blocks = (int)std::min<int64_t>(1024, ((int64_t)sg.m.size() + 255) / 256);
-            k_roots<<<std::max(1, blocks), 256>>>(sg.n, FFT3_FORWARD, d_m, (int64_t)sg.m.size(),
-                                                  fp64 ? (double *)P->d_tw + 2 * sg.off : nullptr,
-                                                  fp64 ? nullptr : P->d_tw + sg.off);
-            if (fp64)
-                k_roots_fix<<<std::max(1, blocks), 256>>>(
-                    sg.n, d_m, (int64_t)sg.m.size(),
-                    (root62 *)((double2 *)P->d_tw + twiddle_slots(s) + sg.off));
-            e = cudaGetLastError();
-        }
-        if (e != cudaSuccess) {
-            cudaFree(d_m);
-            return fail(FFT3_ERR_CUDA, std::string("twiddle generation: ") + cudaGetErrorString(e));
-        }
+        if (e != cudaSuccess)
+            break;
+        int blocks = (int)std::min<int64_t>(1024, ((int64_t)sg.m.size() + 255) / 256);
+        k_roots<<<std::max(1, blocks), 256>>>(sg.n, FFT3_FORWARD, d_m + sg.off, (int64_t)sg.m.size(),
+                                              fp64 ? (double *)P->d_tw + 2 * sg.off : nullptr,
+                                              fp64 ? nullptr : P->d_tw + sg.off);
+        if (fp64)
+            k_roots_fix<<<std::max(1, blocks), 256>>>(sg.n, d_m + sg.off, (int64_t)sg.m.size(),
+                                                      (root62 *)((double2 *)P->d_tw + twiddle_slots(s) + sg.off));
+        e = cudaGetLastError();
     }
-    cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess)
+        e = cudaDeviceSynchronize();
     cudaFree(d_m);
     if (e != cudaSuccess)
         return fail(FFT3_ERR_CUDA, std::string("twiddle generation: ") + cudaGetErrorString(e));
