@@ -17,11 +17,11 @@
 // before anything has been stored.
 //
 // What bounds it: latency at 16 warps per SM (128 registers: 16 values of four
-// words each) and the integer pipe, 48% busy; the FP64 pipe carries only half of
-// the final roundings.  256^3: 580 us, 2.8 TB/s per pass, against 2502 us with
+// words each); the ALU pipe is 57% busy, issue 52%; the FP64 pipe carries only half
+// of the final roundings.  256^3: 579 us, 2.8 TB/s per pass, against 2502 us with
 // FP64 stages (2 lanes per clock and SM); without the shifts up, which dominated
-// lines need, 567.  Tried: radix-8 plans (24 warps, one
-// exchange more) 671 us; up to 168 registers (12 warps) 630 us.
+// lines need, 565.  Tried: radix-8 plans (24 warps, one exchange more) 671 us; up
+// to 168 registers (12 warps) 630 us.
 // The runtime-radix kernel (k_pass_g64) covers the other lengths.
 #pragma once
 
