@@ -31,13 +31,15 @@
 // first stage or over more than 2048 points from radix 5 on, are too coarse for
 // spikes over a background: there every first-stage butterfly must hold a value of
 // 2^-4 of the largest (fix_strict).
+// What is given up: results that are small because larger values cancel exactly are
+// good to about 2^-57 of the line's largest value, where FP64 may hold more bits of them.
 // Measured on the host over every radix list of the plans (relative 2-norm per line
 // against long double; flat, real, tones, bumps, spectra, constants and spikes over
 // a background of 10^-1 to 10^-12): on the lines taken at most the error of the same
 // stages in FP64: flat lines 0.5e-16 against 2.9e-16, the hardest (4096 points, a
-// spike over 10^-12) 2.1e-16 against 2.4e-16.  With shifts up after the first stage
-// of some lists alone that spike had 5e-16 and more, and one over 1e-3 had 1.1e-15 at
-// 256 points as 8 x 8 x 4.
+// spike over 10^-12) 2.1e-16 against 2.4e-16.  A shift up after the first stage of
+// lines from 512 points on alone left a spike over 1e-3 with 1.1e-15 at 256 points
+// as 8 x 8 x 4.
 // Other lines, and those with an infinity, a NaN or values so large or small
 // that their exponent cannot be carried (below 2^-895, above 2^1007), take the
 // FP64 stages.
