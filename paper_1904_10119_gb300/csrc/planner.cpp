@@ -1278,18 +1278,17 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
     // Buffers are asked to be 16-byte aligned, but plans without TMA run on 8 bytes.
     // A streamed pass that took the place of a kernel with plain loads keeps that
     // kernel for such an input: `make` plans the pass without streaming.
-    auto keep_unaligned = [&](PassPlan *p, auto make) -> int {
+    // (Where that cannot be planned, such an input is refused.)
+    auto keep_unaligned = [&](PassPlan *p, auto make) {
         if (p->kind != PK_CSTREAM)
-            return FFT3_OK;
+            return;
         PassPlan q;
         s.no_stream = true;
-        const int r = make(&q);
-        s.no_stream = false;
-        if (!r) {
+        if (make(&q) == FFT3_OK) {
             p->unaligned = (int)s.unaligned.size();
             s.unaligned.push_back(q);
         }
-        return r;
+        s.no_stream = false;
     };
     auto add_nat = [&](int d, bool unaligned = false) -> int {
         if (ns[d] == 1)
@@ -1300,10 +1299,10 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
             return make_line_pass(&s, d, ns[d], geom_natural(d, n0, n1, n2, batch), false, from, BUF_OUT, q, err);
         };
         int r = make(&p);
-        if (!r && unaligned)
-            r = keep_unaligned(&p, make);
         if (r)
             return r;
+        if (unaligned)
+            keep_unaligned(&p, make);
         s.passes.push_back(p);
         cur = BUF_OUT;
         return FFT3_OK;
@@ -1567,7 +1566,7 @@ int build_schedule(int n0, int n1, int n2, int batch, int dtype, int decomp, int
                 auto make = [&](PassPlan *v) { return make_vol_pass(&s, d, ns[d], p, g, cur, BUF_OUT, v, err); };
                 rc = make(&q);
                 if (!rc && ns[d] < 512) // k_volc and k_vol take these lengths with plain loads
-                    rc = keep_unaligned(&q, make);
+                    keep_unaligned(&q, make);
             }
             if (rc)
                 return rc;

@@ -98,8 +98,8 @@ def test_lines_left_to_fp64(n):
                 np.abs(a - b).max() <= 5e-324 * 4 * n
 
 
-@pytest.mark.parametrize("order", range(4))
-@pytest.mark.parametrize("n", [48, 64, 120, 128, 256, 375, 512, 600, 1024, 2048])
+@pytest.mark.parametrize("order", range(5))
+@pytest.mark.parametrize("n", [48, 64, 120, 128, 256, 375, 512, 600, 1024, 2048, 2560])
 def test_dominated_lines_keep_fp64_accuracy(n, order):
     """One value just above a power of two over a small background, and its
     transform (a constant with noise), under every radix order: no further off
